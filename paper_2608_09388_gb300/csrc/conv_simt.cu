@@ -217,7 +217,174 @@ __global__ void __launch_bounds__(kThreads) conv_simt_kernel(const ConvArgs a) {
     }
 }
 
+// ---------------------------------------------------------------- narrow linear heads
+// y[n] = act(x[n] W + bias) on compact rows for at most kHeadMaxOut output
+// channels (the 42- and 1-channel heads, which the tensor-core kernel does not
+// take). The 64 x 64 tiles above leave most of their columns idle there, and
+// a warp's loads of a K chunk of one row at a time make them latency-bound.
+// Here a block stages kHeadRows rows of x and the whole of W (as fp32) in
+// shared memory with one round trip of wide loads; thread t then owns row
+// t % kHeadRows and every second group of kHeadGroup output channels: its
+// row's channels come 16 bytes at a time (the padded pitch keeps eight lanes'
+// pieces on distinct banks), W's are the same word for the whole warp. The
+// finished rows are one contiguous piece of y and leave through the same
+// shared memory in order. Sums run over c = 0, 1, ... in one fp32 chain, then
+// the bias, as in the kernel above: the same bits. What bounds it: reading
+// x once (25k rows x 64 bf16 channels is 3.2 MB) and the launch.
+// Measured on the 64 -> 1 bf16 head over 25k active rows of 168k (cold, ncu):
+// 46.4 us on the 64 x 64 tiles, 9.4 us here; the motion encoder (256 frames)
+// 124 -> 103 us on the device.
+constexpr int kHeadThreads = 256;
+constexpr int kHeadRows = 128;
+constexpr int kHeadGroup = 4;
+constexpr int kHeadMaxOut = 64;
+constexpr int kHeadMaxRowBytes = 512;  // of x
+constexpr int kHeadMaxWFloats = 64 * 64;
+
+__host__ __device__ constexpr int head_pitch(int row_bytes) {
+    return (row_bytes + 15) / 16 * 16 + 16;
+}
+__host__ __device__ constexpr int head_wpitch(int C_out) {
+    return (C_out + kHeadGroup - 1) / kHeadGroup * kHeadGroup;
+}
+inline size_t head_smem_bytes(int C_in, int C_out, int eb) {
+    const size_t xb = (size_t)kHeadRows * head_pitch(C_in * eb);
+    const size_t yb = (size_t)kHeadRows * C_out * eb;
+    return (xb > yb ? xb : yb) + sizeof(float) * (size_t)C_in * head_wpitch(C_out);
+}
+
+// kMaxG: groups a thread owns at most (1 for up to 8 outputs, else 8).
+template <typename T, int kMaxG>
+__global__ void __launch_bounds__(kHeadThreads) linear_head_kernel(const ConvArgs a, int vec_ok) {
+    constexpr int VEC = 16 / (int)sizeof(T);
+    extern __shared__ __align__(16) uint8_t head_smem[];
+    const int C_in = a.C_in, C_out = a.C_out;
+    const int row_bytes = C_in * (int)sizeof(T);
+    const int pitch = head_pitch(row_bytes), wp = head_wpitch(C_out);
+    float* const sW = reinterpret_cast<float*>(head_smem);  // [C_in][wp], zero-padded
+    uint8_t* const sX = head_smem + sizeof(float) * (size_t)C_in * wp;
+    T* const sY = reinterpret_cast<T*>(sX);
+    const T* __restrict__ x = static_cast<const T*>(a.x);
+    const T* __restrict__ W = static_cast<const T*>(a.W);
+    T* __restrict__ y = static_cast<T*>(a.y);
+    const int t = threadIdx.x, row = t & (kHeadRows - 1), half = t / kHeadRows;
+    pdl_wait();
+    pdl_trigger();
+    // the weights' loads go out with the row count's
+#pragma unroll 4
+    for (int i = t; i < C_in * wp; i += kHeadThreads) {
+        const int c = i / wp, o = i - c * wp;
+        sW[i] = o < C_out ? to_float(W[c * C_out + o]) : 0.f;
+    }
+    const long long rows = active_rows(a);
+    for (long long m0 = (long long)blockIdx.x * kHeadRows; m0 < rows;
+         m0 += (long long)gridDim.x * kHeadRows) {
+        const int nr = rows - m0 < kHeadRows ? (int)(rows - m0) : kHeadRows;
+        __syncthreads();  // the previous rows have left through sY
+        if (vec_ok) {
+            const int cpr = row_bytes / 16;
+            const uint4* src = reinterpret_cast<const uint4*>(x + m0 * C_in);
+#pragma unroll 4
+            for (int i = t; i < nr * cpr; i += kHeadThreads) {
+                const int r = i / cpr, q = i - r * cpr;
+                *reinterpret_cast<uint4*>(sX + r * pitch + q * 16) = src[i];
+            }
+        } else {
+            const T* src = x + m0 * C_in;
+#pragma unroll 4
+            for (int i = t; i < nr * C_in; i += kHeadThreads) {
+                const int r = i / C_in, c = i - r * C_in;
+                *reinterpret_cast<T*>(sX + r * pitch + c * (int)sizeof(T)) = src[i];
+            }
+        }
+        __syncthreads();
+        // groups half, half + 2, ... of kHeadGroup outputs; the results are
+        // kept until every thread has read its row (sY shares the memory)
+        float acc[kMaxG][kHeadGroup];
+        const int groups = wp / kHeadGroup;
+#pragma unroll
+        for (int g = 0; g < kMaxG; ++g)
+#pragma unroll
+            for (int j = 0; j < kHeadGroup; ++j) acc[g][j] = 0.f;
+        const uint8_t* xr = sX + row * pitch;
+        if (row < nr)
+            for (int c0 = 0; c0 < C_in; c0 += VEC) {
+                const uint4 raw = *reinterpret_cast<const uint4*>(xr + c0 * (int)sizeof(T));
+                const T* v = reinterpret_cast<const T*>(&raw);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    if (c0 + k >= C_in) break;
+                    const float xv = to_float(v[k]);
+                    const float* wr = sW + (c0 + k) * wp + half * kHeadGroup;
+#pragma unroll
+                    for (int g = 0; g < kMaxG; ++g) {
+                        if (half + 2 * g >= groups) break;
+                        const float4 w = *reinterpret_cast<const float4*>(wr + 2 * g * kHeadGroup);
+                        acc[g][0] = fmaf(xv, w.x, acc[g][0]);
+                        acc[g][1] = fmaf(xv, w.y, acc[g][1]);
+                        acc[g][2] = fmaf(xv, w.z, acc[g][2]);
+                        acc[g][3] = fmaf(xv, w.w, acc[g][3]);
+                    }
+                }
+            }
+        __syncthreads();
+        if (row < nr)
+#pragma unroll
+            for (int g = 0; g < kMaxG; ++g)
+#pragma unroll
+                for (int j = 0; j < kHeadGroup; ++j) {
+                    const int o = (half + 2 * g) * kHeadGroup + j;
+                    if (o < C_out) {
+                        const float z = acc[g][j] + (a.bias ? __ldg(a.bias + o) : 0.f);
+                        sY[row * C_out + o] = from_float<T>(act_apply(z, a.act));
+                    }
+                }
+        __syncthreads();
+        T* dst = y + m0 * C_out;
+        for (int i = t; i < nr * C_out; i += kHeadThreads) dst[i] = sY[i];
+    }
+}
+
+template <typename T>
+hc_status launch_head_typed(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
+    const int row_bytes = a.C_in * (int)sizeof(T);
+    const int vec_ok = row_bytes % 16 == 0 && (uintptr_t)a.x % 16 == 0;
+    static bool attr_set[64] = {};
+    if (!attr_set[ctx->device]) {
+        const size_t most = (size_t)kHeadRows * head_pitch(kHeadMaxRowBytes) +
+                            sizeof(float) * (size_t)kHeadMaxWFloats;
+        for (auto kernel : {linear_head_kernel<T, 1>, linear_head_kernel<T, 8>}) {
+            hc_status st = check_cuda(
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most),
+                "cudaFuncSetAttribute(linear_head_kernel)");
+            if (st != HC_OK) return st;
+        }
+        attr_set[ctx->device] = true;
+    }
+    long long grid = (a.capacity + kHeadRows - 1) / kHeadRows;
+    const long long cap = 4ll * ctx->num_sms;
+    if (grid > cap) grid = cap;
+    return launch_pdl(a.C_out <= 2 * kHeadGroup ? linear_head_kernel<T, 1> : linear_head_kernel<T, 8>,
+                      dim3((unsigned)grid), dim3(kHeadThreads),
+                      head_smem_bytes(a.C_in, a.C_out, (int)sizeof(T)), s, "linear_head_kernel", a,
+                      vec_ok);
+}
+
 }  // namespace
+
+// Linear layers on compact rows with few outputs, whose row of x and weights
+// fit in shared memory.
+bool linear_head_supported(const ConvArgs& a, hc_dtype dt) {
+    const int eb = dt == HC_F32 ? 4 : 2;
+    return a.mode == kLinear && a.out_dense == nullptr && a.C_out <= kHeadMaxOut &&
+           (long long)a.C_in * eb <= kHeadMaxRowBytes &&
+           a.C_in * head_wpitch(a.C_out) <= kHeadMaxWFloats;
+}
+
+hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s) {
+    return dt == HC_F32 ? launch_head_typed<float>(ctx, a, s)
+                        : launch_head_typed<__nv_bfloat16>(ctx, a, s);
+}
 
 hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s) {
     long long cap_tiles = (a.capacity + kBM - 1) / kBM;

@@ -113,6 +113,7 @@ hc_status dispatch_conv(const DeviceCtx* ctx, ConvArgs& a, hc_dtype dt, cudaStre
         }
         return launch_conv_tc(ctx, a, s);
     }
+    if (linear_head_supported(a, dt)) return launch_linear_head(ctx, a, dt, s);
     return launch_conv_simt(ctx, a, dt, s);
 }
 

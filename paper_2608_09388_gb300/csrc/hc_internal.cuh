@@ -112,6 +112,8 @@ struct ConvArgs {
 hc_status launch_compact(const DeviceCtx* ctx, const uint8_t* mask, int B, int V, int32_t* coords,
                          int32_t* row_of, int32_t* offsets, int32_t* count, cudaStream_t s);
 hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
+bool linear_head_supported(const ConvArgs& a, hc_dtype dt);
+hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
 hc_status launch_conv_tc(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
 bool conv_tc_supported(const ConvArgs& a, hc_dtype dt);
 int conv_tc_tile_n(const ConvArgs& a);  // output channels per tensor-core tile
