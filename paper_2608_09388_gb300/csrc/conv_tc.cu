@@ -1254,6 +1254,15 @@ hc_status encode_2d(CUtensorMap* m, const void* base, long long rows, long long 
     return HC_OK;
 }
 
+}  // namespace
+
+hc_status encode_map_2d(CUtensorMap_st* m, const void* base, long long rows, long long cols,
+                        int box_cols, int box_rows) {
+    return encode_2d(m, base, rows, cols, box_cols, box_rows);
+}
+
+namespace {
+
 // The weight matrix [K, C_out] (C_out a multiple of 64) as the 3-D tensor
 // [C_out / 64][K][64] with 128-byte swizzled boxes of 64 x box_k x box_blocks.
 hc_status encode_w3d(CUtensorMap* m, const void* base, long long K, long long C_out, int box_k,

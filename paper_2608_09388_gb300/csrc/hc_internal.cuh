@@ -9,6 +9,8 @@
 
 #include "hc.h"
 
+struct CUtensorMap_st;
+
 namespace hc {
 
 // ------------------------------------------------------------ status bits
@@ -118,6 +120,10 @@ hc_status launch_conv_tc(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s
 bool conv_tc_supported(const ConvArgs& a, hc_dtype dt);
 int conv_tc_tile_n(const ConvArgs& a);  // output channels per tensor-core tile
 size_t conv_tc_pad_bytes(const ConvArgs& a);  // 0 when C_in % 8 == 0
+// 2-D bf16 tensor map of a row-major [rows, cols] matrix, 128-byte swizzled
+// boxes of box_cols x box_rows, zeros outside.
+hc_status encode_map_2d(CUtensorMap_st* m, const void* base, long long rows, long long cols,
+                        int box_cols, int box_rows);
 // Compaction fused with the Eq. 4 mapping (frames of at most 65535 vertices).
 bool compact_map_supported(int B, int V, int L);
 hc_status launch_compact_map(const DeviceCtx* ctx, const uint8_t* mask, int B, int V,
@@ -301,6 +307,12 @@ __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, bool 
 __device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src, bool valid) {
     uint32_t n = valid ? 4u : 0u;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "r"(n)
+                 : "memory");
+}
+// 8 bytes, zero-filled when !valid (both addresses 8-byte aligned).
+__device__ __forceinline__ void cp_async_8(uint32_t dst, const void* src, bool valid) {
+    uint32_t n = valid ? 8u : 0u;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "r"(n)
                  : "memory");
 }
 // Arrive on `bar` once every cp.async issued so far by this thread has
