@@ -5,22 +5,28 @@
 //   dbias[o]  = sum_n dz[n][o]
 //   dW[l*C_in + c][o] = sum_n x[j(n,l)][c] * dz[n][o]
 //   dx[j][c]  = sum over taps (n, l) reading j of (dz[n] W_l^T)[c]
-// Kernels (every sum in a fixed order, no floating-point atomics):
+// Most taps of a sparse mask are absent, so every contraction runs over the
+// present taps (n, l) only, gathered slot by slot. Kernels (every sum in a
+// fixed order, no floating-point atomics):
 //   act_bwd_kernel      dz (stored in the layer dtype) and per-block column
 //                       sums of dz in fp32 (act_bwd_vec_kernel: 16-byte
-//                       chunks); dbias_kernel adds the blocks.
-//   wgrad (tcgen05)     split-K [L*C_in] x [C_out] tiles: A = the gathered
-//                       input rows (cp.async through the rulebook), B = dz,
-//                       both MN-major, fp32 accumulators in TMEM; fp32 on
-//                       CUDA cores otherwise. wgrad_reduce adds the splits.
-//   dgrad               P = dz W^T by the linear conv kernels (W^T
-//                       materialised once), then every input row sums the P
-//                       slices of the taps that read it, in (n, l) order,
-//                       from the transposed mapping (rb_* kernels: counts,
-//                       exclusive scan, fill, per-row sort): a block per
-//                       range of rows, their keys staged in shared memory,
-//                       where rows are whole 16-byte chunks.
+//                       chunks); further blocks of the same launch count the
+//                       present taps per (slot, row unit) for wgrad and the
+//                       taps of the transposed mapping per slot for dgrad.
+//   wgrad               dW_l = sum over the slot's present taps: equal runs
+//                       of taps per CTA, compacted from the rulebook on the
+//                       fly, x and dz rows gathered; tcgen05 (fp32
+//                       accumulators in TMEM) or CUDA cores (fp32).
+//                       bwd_collect adds a slot's runs and dbias's blocks.
+//   dgrad               tap_slots: the taps of the transposed mapping listed
+//                       per slot; tap GEMM: P[e] = dz[n] W_l^T for the e-th
+//                       tap (n, l) of the mapping; seg_sum: every input row
+//                       sums its own, consecutive rows of P, in (n, l) order.
+// The transposed mapping itself: rb_* kernels (counts, exclusive scan, fill,
+// per-row sort).
 #include <cuda_bf16.h>
+
+#include <cuda.h>
 
 #include "hc_internal.cuh"
 
@@ -52,19 +58,122 @@ __device__ __forceinline__ long long clamp_rows(const int32_t* count, long long 
                                                 unsigned* status) {
     long long n = *count;
     if (n < 0) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) report(status, kErrIndex);
+        if (threadIdx.x == 0) report(status, kErrIndex);
         return 0;
     }
     if (n > capacity) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) report(status, kErrCapacity);
+        if (threadIdx.x == 0) report(status, kErrCapacity);
         return capacity;
     }
     return n;
 }
 
+// ---------------------------------------------------------------- tap counts
+// Present taps, counted by the first blocks of the dz launch (they read other
+// inputs than dz and hide behind it):
+//   unit_cnt[l * kUnits + u]  taps of slot l in the row unit u (the rows cut
+//                             into kUnits equal pieces), a warp each: where
+//                             wgrad cuts the present taps into equal runs;
+//   unit_list                 those taps as (j + 1, n + 1) in row order, unit
+//                             u of slot l from entry l * capacity + (its
+//                             first row) on (zeros mean an absent tap);
+//   hist[b * L + l]           taps of slot l in the b-th of hist_blocks equal
+//                             pieces of the transposed mapping: where
+//                             tap_slots places them.
+constexpr int kUnits = 128;
+
+__host__ __device__ inline long long unit_rows(long long rows) {
+    const long long r = (rows + kUnits - 1) / kUnits;
+    return r < 64 ? 64 : r;
+}
+
+struct PrepArgs {
+    int act_blocks, unit_blocks, hist_blocks;  // unit_blocks / hist_blocks: 0 = not wanted
+    const int32_t* rb;
+    int L, x_rows;
+    int32_t* unit_cnt;
+    int2* unit_list;
+    const int32_t* row_ptr;
+    const int32_t* taps;
+    int32_t* hist;
+    unsigned* status;
+};
+
+// Taps of the transposed mapping (the table's end, inside its capacity).
+__device__ __forceinline__ long long total_taps(const int32_t* row_ptr, int x_rows,
+                                                long long capL) {
+    const long long t = __ldg(row_ptr + x_rows);
+    return t < 0 ? 0 : (t > capL ? capL : t);
+}
+// Keys outside [0, capL) count as slot 0 (their row of P is zeros).
+__device__ __forceinline__ int slot_of(int key, int L, long long capL, int& n) {
+    if (key < 0 || key >= capL) {
+        n = -1;
+        return 0;
+    }
+    n = key / L;
+    return key - n * L;
+}
+
+__device__ void count_taps(const PrepArgs& p, const int32_t* count, long long capacity) {
+    const int lane = threadIdx.x & 31;
+    int b = (int)blockIdx.x;
+    if (b < p.unit_blocks) {
+        const int unit = b * 8 + (threadIdx.x >> 5);
+        if (unit >= p.L * kUnits) return;
+        long long rows = *count;
+        rows = rows < 0 ? 0 : (rows > capacity ? capacity : rows);
+        const long long ur = unit_rows(rows);
+        const int l = unit / kUnits, u = unit - l * kUnits;
+        const long long r0 = u * ur, r1 = r0 + ur < rows ? r0 + ur : rows;
+        const int32_t* src = p.rb + l * capacity;
+        int2* dst = p.unit_list + l * capacity + r0;
+        int c = 0;
+        unsigned err = 0;
+        for (long long r = r0; r < r1; r += 256) {
+            int j[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const long long n = r + 32 * q + lane;
+                j[q] = n < r1 ? __ldg(src + n) : -1;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const bool on = j[q] >= 0 && j[q] < p.x_rows;
+                if (!on && j[q] != -1) err |= kErrIndex;
+                const unsigned m = __ballot_sync(0xffffffffu, on);
+                if (on)
+                    dst[c + __popc(m & ((1u << lane) - 1u))] =
+                        make_int2(j[q] + 1, (int)(r + 32 * q + lane) + 1);
+                c += __popc(m);
+            }
+        }
+        if (lane == 0) p.unit_cnt[unit] = c;
+        if (err) report(p.status, err);
+        return;
+    }
+    b -= p.unit_blocks;
+    __shared__ int s_hist[HC_MAX_SPIRAL];
+    if (threadIdx.x < HC_MAX_SPIRAL) s_hist[threadIdx.x] = 0;
+    __syncthreads();
+    const long long capL = capacity * p.L;
+    const long long T = total_taps(p.row_ptr, p.x_rows, capL);
+    const long long E = (T + p.hist_blocks - 1) / p.hist_blocks;
+    const long long e0 = b * E, e1 = e0 + E < T ? e0 + E : T;
+    for (long long e = e0 + threadIdx.x; e - lane < e1; e += 256) {
+        const bool in = e < e1;
+        int n;
+        const int l = in ? slot_of(__ldg(p.taps + e), p.L, capL, n) : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, l);
+        if (in && lane == __ffs(same) - 1) atomicAdd(&s_hist[l], __popc(same));
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < p.L) p.hist[b * p.L + threadIdx.x] = s_hist[threadIdx.x];
+}
+
 // ---------------------------------------------------------------- dz, dbias
 // Block (64, 4): thread (tx, ty) takes columns g*64 + tx of rows r0 + ty +
-// 4 i of the block's row chunks (chunks blockIdx.x, + gridDim.x, ...); the
+// 4 i of the block's row chunks (chunks blockIdx.x, + prep.act_blocks, ...); the
 // four row lanes' sums meet in shared memory and the block writes one
 // partial per column.
 constexpr int kActRowsPerBlock = 16;
@@ -73,18 +182,23 @@ template <typename T>
 __global__ void __launch_bounds__(256)
     act_bwd_kernel(const T* __restrict__ y, const T* __restrict__ dy, const int32_t* count,
                    long long capacity, int C_out, int act, T* __restrict__ dz,
-                   float* __restrict__ bpart, unsigned* status) {
+                   float* __restrict__ bpart, const PrepArgs prep, unsigned* status) {
     __shared__ float red[4][64];
     pdl_wait();
     pdl_trigger();
+    if ((int)blockIdx.x < prep.unit_blocks + prep.hist_blocks) {
+        count_taps(prep, count, capacity);
+        return;
+    }
+    const int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
     const long long rows = clamp_rows(count, capacity, status);
     const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     for (int g0 = 0; g0 < C_out; g0 += 64) {
         const int o = g0 + tx;
         float sum = 0.f;
         if (o < C_out)
-            for (long long r0 = (long long)blockIdx.x * kActRowsPerBlock; r0 < rows;
-                 r0 += (long long)gridDim.x * kActRowsPerBlock) {
+            for (long long r0 = (long long)block * kActRowsPerBlock; r0 < rows;
+                 r0 += (long long)prep.act_blocks * kActRowsPerBlock) {
                 const long long r1 = r0 + kActRowsPerBlock < rows ? r0 + kActRowsPerBlock : rows;
                 for (long long rb0 = r0 + ty; rb0 < r1; rb0 += 16) {
                     // four rows' loads in flight, then their arithmetic
@@ -111,14 +225,14 @@ __global__ void __launch_bounds__(256)
         red[ty][tx] = sum;
         __syncthreads();
         if (ty == 0 && o < C_out)
-            bpart[(long long)blockIdx.x * C_out + o] = ((red[0][tx] + red[1][tx]) + red[2][tx]) + red[3][tx];
+            bpart[(long long)block * C_out + o] = ((red[0][tx] + red[1][tx]) + red[2][tx]) + red[3][tx];
         __syncthreads();
     }
 }
 
 // Vectorised dz for rows of 16-byte chunks (cpr = C_out / VEC of them,
 // cpr dividing 256): a block takes kActVecItems / cpr consecutive rows
-// (ranges blockIdx.x, + gridDim.x, ...); thread t always holds chunk
+// (ranges block, + prep.act_blocks, ...); thread t always holds chunk
 // t % cpr, so it sums its VEC columns over its rows in registers, and the
 // 256 / cpr row lanes of a column meet in shared memory in a fixed order.
 constexpr int kActVecItems = 1024;
@@ -127,12 +241,17 @@ template <typename T>
 __global__ void __launch_bounds__(256)
     act_bwd_vec_kernel(const T* __restrict__ y, const T* __restrict__ dy, const int32_t* count,
                        long long capacity, int C_out, int act, T* __restrict__ dz,
-                       float* __restrict__ bpart, unsigned* status) {
+                       float* __restrict__ bpart, const PrepArgs prep, unsigned* status) {
     constexpr int VEC = 16 / sizeof(T);
     constexpr int kPer = kActVecItems / 256;
     __shared__ float red[256 * VEC];
     pdl_wait();
     pdl_trigger();
+    if ((int)blockIdx.x < prep.unit_blocks + prep.hist_blocks) {
+        count_taps(prep, count, capacity);
+        return;
+    }
+    const int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
     const long long rows = clamp_rows(count, capacity, status);
     const int t = threadIdx.x;
     const int cpr = C_out / VEC, lanes = 256 / cpr;
@@ -141,7 +260,7 @@ __global__ void __launch_bounds__(256)
     float sum[VEC];
 #pragma unroll
     for (int k = 0; k < VEC; ++k) sum[k] = 0.f;
-    for (long long r0 = (long long)blockIdx.x * R; r0 < rows; r0 += (long long)gridDim.x * R) {
+    for (long long r0 = (long long)block * R; r0 < rows; r0 += (long long)prep.act_blocks * R) {
         uint4 yv[kPer], gv[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
@@ -178,47 +297,7 @@ __global__ void __launch_bounds__(256)
     for (int o = t; o < C_out; o += 256) {
         float s = 0.f;
         for (int j = 0; j < lanes; ++j) s += red[j * C_out + o];
-        bpart[(long long)blockIdx.x * C_out + o] = s;
-    }
-}
-
-// dbias: block (32, 32) per 32 columns; row lane ty adds partials ty,
-// ty + 32, ... and the 32 lane sums are added in order.
-__global__ void dbias_kernel(const float* __restrict__ bpart, int nblocks, int C_out,
-                             float* __restrict__ dbias) {
-    __shared__ float red[32][33];
-    pdl_wait();
-    pdl_trigger();
-    const int o = blockIdx.x * 32 + threadIdx.x;
-    float s = 0.f;
-    if (o < C_out)
-#pragma unroll 4
-        for (int b = threadIdx.y; b < nblocks; b += 32) s += bpart[(long long)b * C_out + o];
-    red[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0 && o < C_out) {
-        float t = 0.f;
-#pragma unroll 8
-        for (int i = 0; i < 32; ++i) t += red[i][threadIdx.x];
-        dbias[o] = t;
-    }
-}
-
-// W [K, C_out] -> W^T [C_out, K]
-template <typename T>
-__global__ void transpose_kernel(const T* __restrict__ W, int K, int C_out, T* __restrict__ Wt) {
-    __shared__ T tile[32][33];
-    pdl_wait();
-    pdl_trigger();
-    const int k0 = blockIdx.y * 32, o0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int k = k0 + i, o = o0 + threadIdx.x;
-        if (k < K && o < C_out) tile[i][threadIdx.x] = W[(long long)k * C_out + o];
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int o = o0 + i, k = k0 + threadIdx.x;
-        if (k < K && o < C_out) Wt[(long long)o * K + k] = tile[threadIdx.x][i];
+        bpart[(long long)block * C_out + o] = s;
     }
 }
 
@@ -443,93 +522,146 @@ __global__ void __launch_bounds__(kSortRows)
     }
 }
 
-// ---------------------------------------------------------------- dgrad gather-sum
-// dx[j][c] = sum over the taps e of row j (ascending n*L + l) of
-// P[n][l*C_in + c]; U-sized chunks of VEC elements; rows without taps get 0.
-// Keys are checked against the P rows that exist (n < capacity) and the
-// row ranges against the taps table (a malformed table is reported and its
-// entries skipped).
-template <typename T, typename U>
-__global__ void dgrad_kernel(const T* __restrict__ P, const int32_t* __restrict__ ptr,
-                             const int32_t* __restrict__ taps, int x_rows, int L, int C_in,
-                             long long capacity, T* __restrict__ dx, unsigned* status) {
-    constexpr int VEC = sizeof(U) / sizeof(T);
-    pdl_wait();
-    pdl_trigger();
-    const int cpr = C_in / VEC;
-    const long long total = (long long)x_rows * cpr;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        int ci;
-        const long long j = div32(i, cpr, ci);
-        const int c = ci * VEC;
-        float acc[VEC];
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
-        int a = __ldg(ptr + j), b = __ldg(ptr + j + 1);
-        if (a < 0 || b < a || (long long)b > capacity * L) {
-            if (c == 0) report(status, kErrIndex);
-            b = a;
-        }
-        // a batch of keys, then all their P chunks in flight, then the sums
-        // (in key order)
-        constexpr int kBatchTaps = 4;
-        for (int e0 = a; e0 < b; e0 += kBatchTaps) {
-            int key[kBatchTaps];
-#pragma unroll
-            for (int i = 0; i < kBatchTaps; ++i) key[i] = e0 + i < b ? __ldg(taps + e0 + i) : -1;
-            U raw[kBatchTaps];
-#pragma unroll
-            for (int i = 0; i < kBatchTaps; ++i) {
-                if (e0 + i >= b) continue;
-                if (key[i] < 0 || (long long)key[i] >= capacity * L) {
-                    if (c == 0) report(status, kErrIndex);
-                    key[i] = -1;
-                    continue;
-                }
-                // key n*L + l: P's row n, slot l starts at (n*L + l)*C_in
-                raw[i] = *reinterpret_cast<const U*>(P + (long long)key[i] * C_in + c);
-            }
-#pragma unroll
-            for (int i = 0; i < kBatchTaps; ++i) {
-                if (e0 + i >= b || key[i] < 0) continue;
-                const T* v = reinterpret_cast<const T*>(&raw[i]);
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) acc[k] += to_f(v[k]);
-            }
-        }
-        U out;
-        T* ov = reinterpret_cast<T*>(&out);
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) ov[k] = from_f<T>(acc[k]);
-        *reinterpret_cast<U*>(dx + j * C_in + c) = out;
-    }
-}
-
 // ---------------------------------------------------------------- wgrad
+// dW_l[c][o] = sum over the present taps (n, j) of slot l of x[j][c] dz[n][o].
+// The present taps of all slots, slot by slot and in row order, are one list
+// of T positions; CTA g of G takes positions [g Q, (g + 1) Q), Q = T / G
+// rounded up to kBK, whatever slots and rows they fall into (its "segments":
+// one per slot it touches). Cutting by taps and not by rows keeps the CTAs
+// even although slot 0 (the vertex itself) is always present and the others
+// are as dense as the mask. A segment's sum goes to partial g + l: within a
+// CTA l rises, and a later CTA starts at the slot where the one before it
+// ended, so no two segments share one, and G + L partials suffice.
 constexpr int kTile = 128;
 constexpr int kBK = 64;
-constexpr int kStages = 6;
-constexpr int kOpBytes = kBK * kTile * 2;
-constexpr int kProducerWarps = 4, kEpilogueWarps = 4;
-constexpr int kMmaWarp = kProducerWarps + kEpilogueWarps;
-constexpr int kThreadsTc = (kMmaWarp + 1) * 32;
-constexpr int kPartElems = kTile * kTile;
-constexpr size_t kSmemTc = 1024 + (size_t)kStages * 2 * kOpBytes + 256;
-// kind::f16: D fp32, A and B bf16, both MN-major, N = 128, M = 128.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                            ((uint32_t)(kTile >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
 
 struct WgradArgs {
     const void* x;
-    const int32_t* rb;
     const int32_t* count;
     const void* dz;
     long long capacity;
-    int x_rows, L, C_in, C_out, K;  // K = L * C_in
-    int m_tiles, n_tiles, T, splits;  // rows split on the device, from *count
-    float* part;                      // [splits * T][128][128]
+    int L, C_in, C_out;
+    int c_tiles, o_tiles, G;     // grid: G x (c_tiles * o_tiles)
+    const int32_t* unit_cnt;     // [L][kUnits]
+    const int2* unit_list;       // [L][capacity]
+    int32_t* slot_pos;           // [L + 2]: first position of each slot, T, Q (for the reduction)
+    float* part;                 // [c_tiles * o_tiles][G + L][BC][kTile]
     unsigned* status;
+};
+
+// Positions of the units: s_pre[i] = present taps before unit i of the [L][kUnits]
+// list, s_pre[L * kUnits] = T, by the first 256 threads of the block (the
+// caller synchronises after it). red: 8 ints.
+__device__ __forceinline__ void unit_positions(const int32_t* __restrict__ cnt, int n, int* s_pre,
+                                               int* red) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (n + 255) / 256;
+    int sum = 0;
+    if (t < 256)
+        for (int i = t; i < n; i += 256) s_pre[i] = __ldg(cnt + i);
+    __syncthreads();
+    int own[HC_MAX_SPIRAL * kUnits / 256];
+    if (t < 256) {
+#pragma unroll
+        for (int q = 0; q < HC_MAX_SPIRAL * kUnits / 256; ++q) {
+            const int i = t * per + q;
+            own[q] = q < per && i < n ? s_pre[i] : 0;
+            sum += own[q];
+        }
+    }
+    int x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (t < 256 && lane == 31) red[warp] = x;
+    __syncthreads();
+    if (t < 256) {
+        int run = x - sum;
+        for (int w = 0; w < warp; ++w) run += red[w];
+#pragma unroll
+        for (int q = 0; q < HC_MAX_SPIRAL * kUnits / 256; ++q) {
+            const int i = t * per + q;
+            if (q < per && i < n) s_pre[i] = run;
+            run += own[q];
+        }
+        if (t == 255) s_pre[n] = run;
+    }
+}
+
+// The run of a CTA: positions [p0, p1), and its segments in order.
+struct Run {
+    const int* s_pre;
+    int L;
+    long long p0, p1;
+    __device__ __forceinline__ Run(const int* pre, int L_, int G, int g) : s_pre(pre), L(L_) {
+        const long long T = pre[L_ * kUnits];
+        const long long Q = ((T + G - 1) / G + kBK - 1) / kBK * kBK;
+        p0 = g * Q;
+        p1 = p0 + Q < T ? p0 + Q : T;
+    }
+    // The segment at position pos < p1: its slot (l = the slot of an earlier
+    // position, or 0) and its end.
+    __device__ __forceinline__ long long segment(long long pos, int& l) const {
+        while (s_pre[(l + 1) * kUnits] <= pos) ++l;
+        const long long end = s_pre[(l + 1) * kUnits];
+        return end < p1 ? end : p1;
+    }
+    // Entry of the unit lists (see count_taps) of position pos of slot l.
+    __device__ __forceinline__ long long entry(int l, int pos, long long urows,
+                                               long long capacity) const {
+        int lo = l * kUnits, hi = (l + 1) * kUnits - 1;  // last unit with s_pre <= pos
+#pragma unroll
+        for (int step = 0; step < 7; ++step) {
+            const int mid = (lo + hi + 1) >> 1;
+            const bool le = s_pre[mid] <= pos;
+            lo = le ? mid : lo;
+            hi = le ? hi : mid - 1;
+        }
+        return l * capacity + (lo - l * kUnits) * urows + (pos - s_pre[lo]);
+    }
+};
+static_assert(kUnits == 1 << 7, "Run::entry halves a slot's units seven times");
+
+// tcgen05: D[o][c] (M = 128 output channels of dz, N = BC channels of x),
+// both operands MN-major as gathered: per stage kBK taps, dz's rows as up to
+// two and x's as BC / 64 atoms of 64 channels (kBK rows x 128 bytes each,
+// 128-byte swizzle). What bounds it is the gather: a stage moves up to 32 KB
+// for 2.1 MFLOP. Warp 9 (index) copies the taps' (j, n) from
+// the unit lists into tables of kBK for the producers, up to kQueue ahead, by
+// cp.async, so that no lookup's latency is on the gather's path. (Compacting
+// the rulebook in this warp instead kept the gather waiting for 20 of 58 us
+// at 25% density: the scan's shared-memory accesses queue behind the
+// producers' copies.) Warps 0-3 gather
+// with 16-byte cp.async, warp 8 issues the MMAs, warps 4-7 move a finished
+// segment's sums from TMEM to its partial while the next one accumulates.
+// 167k rows, 9 slots, 128 -> 128, 25% present: 146 -> 45 us (two thirds of the
+// taps were multiplied as zeros, the lookups' latency was paid per stage);
+// 16.4k rows, 12 slots, 64 -> 128, 84% present: 17.5 -> 18.9 us (the rows of
+// dz are gathered per slot, 24 KB a stage). fp32, 25k rows, 9 slots, 64 -> 128,
+// 24% present: 374 -> 31 us. All cold under ncu.
+constexpr int kQueue = 8;
+constexpr int kProducerWarps = 4, kEpilogueWarps = 4;
+constexpr int kMmaWarp = kProducerWarps + kEpilogueWarps;
+constexpr int kIndexWarp = kMmaWarp + 1;
+constexpr int kThreadsTc = (kIndexWarp + 1) * 32;
+constexpr int kAtomBytes = kBK * 128;  // 64 channels of kBK rows
+
+template <int BC>
+struct WgradCfg {
+    static constexpr int kStageBytes = (2 + BC / 64) * kAtomBytes;
+    static constexpr int kStages = BC == 64 ? 8 : 6;
+    static constexpr uint32_t kTmemCols = 2 * BC;
+    static constexpr int kBars = 2 * kStages + 2 * kQueue + 5;
+    static constexpr int kMisc = kStages * kStageBytes;  // barriers, tmem address, abort flag, scan
+    static constexpr int kTables = kMisc + (8 * kBars + 16 + 32 + 127) / 128 * 128;
+    static constexpr int kPre = kTables + kQueue * kBK * 8;
+    // kind::f16: D fp32, A and B bf16, both MN-major, N = BC, M = 128
+    static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) |
+                                       (1u << 16) | ((uint32_t)(BC >> 3) << 17) |
+                                       ((uint32_t)(kTile >> 4) << 24);
+    static size_t smem_bytes(int L) { return 1024 + kPre + sizeof(int) * ((size_t)L * kUnits + 1); }
 };
 
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
@@ -537,41 +669,49 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uin
            ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
-// Warps 0-3 load a stage: thread t owns 16-byte chunk column t % 16 of the
-// tile's 128 columns (of the gathered rows for A, of dz for B) and rows
-// t / 16 + 8 i; the rulebook entries of the next stage are loaded while the
-// current stage's copies go out. Warp 8 issues the MMAs, warps 4-7 write
-// the finished tile to the workspace.
+template <int BC>
 __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs a) {
-    constexpr uint32_t kArrivals = kProducerWarps * 32;
-    constexpr int kRowsPer = kBK / 8;  // rows of a stage per producer thread
+    using C = WgradCfg<BC>;
+    constexpr int kStages = C::kStages;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* const base_ptr = smem_raw + (base - raw);
-    const uint32_t sA = base, sB = base + kStages * kOpBytes;
-    const uint32_t sBar = sB + kStages * kOpBytes;
+    const uint32_t sBar = base + C::kMisc;
     auto full_bar = [&](int s) { return sBar + 8u * s; };
     auto empty_bar = [&](int s) { return sBar + 8u * (kStages + s); };
-    const uint32_t tfull_bar = sBar + 8u * (2 * kStages);
-    const uint32_t fin_bar = sBar + 8u * (2 * kStages + 1);
-    uint8_t* const misc = base_ptr + (sBar - base) + 8 * (2 * kStages + 2);
+    auto qfull_bar = [&](int q) { return sBar + 8u * (2 * kStages + q); };
+    auto qempty_bar = [&](int q) { return sBar + 8u * (2 * kStages + kQueue + q); };
+    auto tfull_bar = [&](int i) { return sBar + 8u * (2 * kStages + 2 * kQueue + i); };
+    auto tempty_bar = [&](int i) { return sBar + 8u * (2 * kStages + 2 * kQueue + 2 + i); };
+    const uint32_t fin_bar = sBar + 8u * (2 * kStages + 2 * kQueue + 4);
+    uint8_t* const misc = base_ptr + C::kMisc + 8 * C::kBars;
     volatile uint32_t* const tmem_holder = reinterpret_cast<volatile uint32_t*>(misc);
     volatile int* const abort_flag = reinterpret_cast<volatile int*>(misc + 4);
+    int* const red = reinterpret_cast<int*>(misc + 16);
+    int* const s_pre = reinterpret_cast<int*>(base_ptr + C::kPre);
+    const uint32_t tables = base + C::kTables;  // [kQueue][kBK] (j, n)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(full_bar(s), kArrivals);
+            mbar_init(full_bar(s), kProducerWarps * 32);
             mbar_init(empty_bar(s), 1);
         }
-        mbar_init(tfull_bar, 1);
+        for (int q = 0; q < kQueue; ++q) {
+            mbar_init(qfull_bar(q), 32);
+            mbar_init(qempty_bar(q), kProducerWarps * 32);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(tfull_bar(i), 1);
+            mbar_init(tempty_bar(i), kEpilogueWarps * 32);
+        }
         mbar_init(fin_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(smem_u32((const void*)tmem_holder), kTile);
+        tmem_alloc(smem_u32((const void*)tmem_holder), C::kTmemCols);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -583,359 +723,1005 @@ __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs
 
     long long rows = *a.count;
     rows = rows < 0 ? 0 : (rows > a.capacity ? a.capacity : rows);
-    const int item = blockIdx.x;
-    const int split = item / a.T;
-    const int tile = item - split * a.T;
-    const int tm = tile / a.n_tiles, tn = tile - tm * a.n_tiles;
-    // the active rows (known on the device) split evenly, in kBK blocks
-    const long long rps = ((rows + a.splits - 1) / a.splits + kBK - 1) / kBK * kBK;
-    const long long r_begin = (long long)split * rps;
-    long long r_end = r_begin + rps;
-    if (r_end > rows) r_end = rows;
-    const int num_kb = r_end > r_begin ? (int)((r_end - r_begin + kBK - 1) / kBK) : 0;
+    unit_positions(a.unit_cnt, a.L * kUnits, s_pre, red);
+    __syncthreads();
+    const int g = blockIdx.x;
+    const int ct = (int)blockIdx.y % a.c_tiles, ot = (int)blockIdx.y / a.c_tiles;
+    const Run run(s_pre, a.L, a.G, g);
+    if (g == 0 && blockIdx.y == 0 && (int)threadIdx.x <= a.L + 1) {
+        const int T = s_pre[a.L * kUnits];
+        a.slot_pos[threadIdx.x] = (int)threadIdx.x <= a.L
+                                      ? s_pre[threadIdx.x * kUnits]
+                                      : ((T + a.G - 1) / a.G + kBK - 1) / kBK * kBK;
+    }
 
     if (warp < kProducerWarps) {
         const __nv_bfloat16* __restrict__ x = static_cast<const __nv_bfloat16*>(a.x);
         const __nv_bfloat16* __restrict__ dz = static_cast<const __nv_bfloat16*>(a.dz);
         const int t = threadIdx.x;
-        const int cc = t & 15, atom = cc >> 3, q = cc & 7;
-        const int m = tm * kTile + cc * 8;  // A column: tap slot l, channel c
-        const bool m_ok = m < a.K;
-        const int l = m_ok ? m / a.C_in : 0, c = m - l * a.C_in;
-        const int32_t* rbl = a.rb + (long long)l * a.capacity;
-        const int o = tn * kTile + cc * 8;  // B column: output channel
-        const bool o_ok = o < a.C_out;
-        unsigned err = 0;
-        int jn[kRowsPer];
-        auto load_taps = [&](int kb, int (&j)[kRowsPer]) {
+        // dz: 16-byte chunk t % 16 of rows t / 16 + 8 i; x: the same, or with
+        // one atom chunk t % 8 of rows t / 8 + 16 i. Columns past the
+        // channels are left as they are (their sums are never stored).
+        constexpr int kXc = BC / 8, kXrows = kProducerWarps * 32 / kXc, kXper = kBK / kXrows;
+        const int zc = t & 15, zr = t >> 4;
+        const int xc = t % kXc, xrow = t / kXc;
+        const int o = ot * kTile + zc * 8, c = ct * BC + xc * 8;
+        const bool o_ok = o < a.C_out, c_ok = c < a.C_in;
+        int st = 0;  // stage and table of the current iteration, and their phases
+        uint32_t ph = 0;
+        int qt = 0;
+        uint32_t qph = 0;
+        bool ok = true;
+        int l = 0;
+        for (long long pos = run.p0; pos < run.p1 && ok;) {
+            const long long end = run.segment(pos, l);
+            for (; pos < end; pos += kBK) {
+                if (!mbar_wait(qfull_bar(qt), qph, abort_flag, a.status)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t tab = tables + (uint32_t)(qt * kBK * 8);
+                int n[8], j[kXper];
 #pragma unroll
-            for (int i = 0; i < kRowsPer; ++i) {
-                const long long n = r_begin + (long long)kb * kBK + (t >> 4) + 8 * i;
-                j[i] = (m_ok && n < r_end) ? __ldg(rbl + n) : -1;
+                for (int i = 0; i < 8; ++i)
+                    n[i] = lds_s32(tab + (uint32_t)(zr + 8 * i) * 8u + 4u) - 1;
+#pragma unroll
+                for (int i = 0; i < kXper; ++i)
+                    j[i] = lds_s32(tab + (uint32_t)(xrow + kXrows * i) * 8u) - 1;
+                mbar_arrive(qempty_bar(qt));
+                if (++qt == kQueue) {
+                    qt = 0;
+                    qph ^= 1u;
+                }
+                if (!mbar_wait(empty_bar(st), ph ^ 1u, abort_flag, a.status)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t z_st = base + st * C::kStageBytes + (zc >> 3) * kAtomBytes;
+                const uint32_t x_st =
+                    base + st * C::kStageBytes + 2 * kAtomBytes + (xc >> 3) * kAtomBytes;
+                if (o_ok)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = zr + 8 * i;
+                        const bool v = n[i] >= 0;
+                        cp_async_16(z_st + r * 128 + (((zc & 7) ^ (r & 7)) << 4),
+                                    dz + (v ? (long long)n[i] * a.C_out + o : 0), v);
+                    }
+                if (c_ok)
+#pragma unroll
+                    for (int i = 0; i < kXper; ++i) {
+                        const int r = xrow + kXrows * i;
+                        const bool v = j[i] >= 0;
+                        cp_async_16(x_st + r * 128 + (((xc & 7) ^ (r & 7)) << 4),
+                                    x + (v ? (long long)j[i] * a.C_in + c : 0), v);
+                    }
+                cp_async_arrive_noinc(full_bar(st));
+                if (++st == kStages) {
+                    st = 0;
+                    ph ^= 1u;
+                }
             }
-        };
-        if (num_kb > 0) load_taps(0, jn);
-        for (int kb = 0; kb < num_kb; ++kb) {
-            int j[kRowsPer];
-#pragma unroll
-            for (int i = 0; i < kRowsPer; ++i) j[i] = jn[i];
-            if (kb + 1 < num_kb) load_taps(kb + 1, jn);
-            const int s = kb % kStages;
-            const uint32_t ph = (uint32_t)((kb / kStages) & 1);
-            if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, a.status)) break;
-            const long long n0 = r_begin + (long long)kb * kBK;
-            const uint32_t a_st = sA + s * kOpBytes + atom * (kBK * 128);
-            const uint32_t b_st = sB + s * kOpBytes + atom * (kBK * 128);
-#pragma unroll
-            for (int i = 0; i < kRowsPer; ++i) {
-                const int r = (t >> 4) + 8 * i;
-                const long long n = n0 + r;
-                const int ji = j[i];
-                if (ji < -1 || ji >= a.x_rows) err |= kErrIndex;
-                const bool av = ji >= 0 && ji < a.x_rows;
-                cp_async_16(a_st + r * 128 + ((q ^ (r & 7)) << 4),
-                            x + (av ? (long long)ji * a.C_in + c : 0), av);
-                const bool bv = o_ok && n < r_end;
-                cp_async_16(b_st + r * 128 + ((q ^ (r & 7)) << 4),
-                            dz + (bv ? n * a.C_out + o : 0), bv);
-            }
-            cp_async_arrive_noinc(full_bar(s));
+            if (pos > end) pos = end;
         }
         cp_async_wait_all();
-        if (err) report(a.status, err);
+    } else if (warp == kIndexWarp) {
+        const long long urows = unit_rows(rows);
+        int qt = 0;
+        uint32_t qph = 0;
+        bool ok = true;
+        int l = 0;
+        for (long long pos = run.p0; pos < run.p1 && ok;) {
+            const long long end = run.segment(pos, l);
+            for (; pos < end; pos += kBK) {
+                // position pos + i -> entry i; zeros past the segment's end
+                long long src[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const long long p = pos + lane + 32 * i;
+                    src[i] = p < end ? run.entry(l, (int)p, urows, a.capacity) : -1;
+                }
+                if (!mbar_wait(qempty_bar(qt), qph ^ 1u, abort_flag, a.status)) {
+                    ok = false;
+                    break;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    cp_async_8(tables + (uint32_t)((qt * kBK + lane + 32 * i) * 8),
+                               a.unit_list + (src[i] >= 0 ? src[i] : 0), src[i] >= 0);
+                cp_async_arrive_noinc(qfull_bar(qt));
+                if (++qt == kQueue) {
+                    qt = 0;
+                    qph ^= 1u;
+                }
+            }
+            pos = end;
+        }
+        cp_async_wait_all();
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
+            int st = 0;
+            uint32_t ph = 0;
+            int seg = 0, l = 0;
             bool ok = true;
-            for (int kb = 0; kb < num_kb; ++kb) {
-                const int s = kb % kStages;
-                const uint32_t ph = (uint32_t)((kb / kStages) & 1);
-                if (!mbar_wait(full_bar(s), ph, abort_flag, a.status)) {
+            for (long long pos = run.p0; pos < run.p1 && ok; ++seg) {
+                const long long end = run.segment(pos, l);
+                const int acc = seg & 1;
+                if (!mbar_wait(tempty_bar(acc), (uint32_t)(((seg >> 1) & 1) ^ 1), abort_flag,
+                               a.status)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                fence_proxy_async_smem();  // operands written by cp.async
-                const uint32_t a_st = sA + s * kOpBytes, b_st = sB + s * kOpBytes;
+                bool first = true;
+                for (; pos < end; pos += kBK) {
+                    if (!mbar_wait(full_bar(st), ph, abort_flag, a.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    fence_proxy_async_smem();  // operands written by cp.async
+                    const uint32_t z_st = base + st * C::kStageBytes, x_st = z_st + 2 * kAtomBytes;
 #pragma unroll
-                for (int k = 0; k < kBK / 16; ++k) {
-                    const uint64_t ad = desc_sw128(a_st + k * 16 * 128, kBK * 128, 1024);
-                    const uint64_t bd = desc_sw128(b_st + k * 16 * 128, kBK * 128, 1024);
-                    tc_mma_bf16(tmem_base, ad, bd, kIdesc, (kb | k) != 0 ? 1u : 0u);
+                    for (int k = 0; k < kBK / 16; ++k) {
+                        const uint64_t zd = desc_sw128(z_st + k * 16 * 128, kAtomBytes, 1024);
+                        const uint64_t xd = desc_sw128(x_st + k * 16 * 128, kAtomBytes, 1024);
+                        tc_mma_bf16(tmem_base + (uint32_t)(acc * BC), zd, xd, C::kIdesc,
+                                    first ? 0u : 1u);
+                        first = false;
+                    }
+                    tc_commit(empty_bar(st));
+                    if (++st == kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
-                tc_commit(empty_bar(s));
+                if (!ok) break;
+                tc_commit(tfull_bar(acc));
+                pos = end;
             }
-            if (ok && num_kb > 0) tc_commit(tfull_bar);
             tc_commit(fin_bar);
             mbar_wait_drain(fin_bar, 0, a.status);
-            if (ok && num_kb == 0) mbar_arrive(tfull_bar);  // empty split: zeros
         }
         __syncwarp();
     } else {
-        const int ew = warp - kProducerWarps;
-        const int row = ew * 32 + lane;
-        float* dst = a.part + (long long)item * kPartElems + (long long)row * kTile;
-        if (mbar_wait(tfull_bar, 0, abort_flag, a.status)) {
+        const int ew = warp - kProducerWarps;  // TMEM lanes 32 ew ..: output channels
+        int seg = 0, l = 0;
+        for (long long pos = run.p0; pos < run.p1; ++seg) {
+            const long long end = run.segment(pos, l);
+            const int acc = seg & 1;
+            if (!mbar_wait(tfull_bar(acc), (uint32_t)((seg >> 1) & 1), abort_flag, a.status)) break;
             tc_fence_after();
+            float* dst = a.part + ((long long)blockIdx.y * (a.G + a.L) + g + l) * (BC * kTile) +
+                         ew * 32 + lane;
 #pragma unroll 1
-            for (int cb = 0; cb < kTile / 32; ++cb) {
+            for (int cb = 0; cb < BC / 32; ++cb) {
                 uint32_t r[32];
-                if (num_kb > 0) {
-                    tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(cb * 32),
-                                       r);
-                    tmem_ld_wait();
-                } else {
+                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(ew * 32) << 16) +
+                                       (uint32_t)(acc * BC + cb * 32),
+                                   r);
+                tmem_ld_wait();
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) r[jj] = 0u;
-                }
-                float4* d4 = reinterpret_cast<float4*>(dst + cb * 32);
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj)
-                    d4[jj] = make_float4(__uint_as_float(r[4 * jj]), __uint_as_float(r[4 * jj + 1]),
-                                         __uint_as_float(r[4 * jj + 2]),
-                                         __uint_as_float(r[4 * jj + 3]));
+                for (int jj = 0; jj < 32; ++jj) dst[(cb * 32 + jj) * kTile] = __uint_as_float(r[jj]);
             }
             tc_fence_before();
+            mbar_arrive(tempty_bar(acc));
+            pos = end;
         }
     }
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTile);
+        tmem_dealloc(tmem_base, C::kTmemCols);
     }
 }
 
-// fp32 (or unaligned bf16) on CUDA cores: 256 threads, 8 x 8 outputs each.
+// CUDA cores (fp32, and bf16 shapes off the tensor cores' alignment): the
+// same runs; a block reads kSimtBatch taps of the lists at a time and
+// multiplies them kSimtBK at a time, the next rows in registers
+// while the current ones are multiplied. 64 channels of x by 128 of dz per
+// block, 4 x 8 per thread: 12 shared-memory words for 32 multiply-adds.
+constexpr int kSimtBK = 16;
+constexpr int kSimtBatch = 256;  // the block's threads: one entry each
+constexpr int kSimtBC = 64;
+
 template <typename T>
-__global__ void __launch_bounds__(256) wgrad_simt_kernel(const WgradArgs a) {
-    constexpr int kBKs = 16;
-    __shared__ float As[kBKs][kTile];
-    __shared__ float Bs[kBKs][kTile];
+__global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
+    __shared__ float Xs[2][kSimtBK][kSimtBC];
+    __shared__ float Zs[2][kSimtBK][kTile];
+    __shared__ int s_j[kSimtBatch], s_n[kSimtBatch], red[8];
+    extern __shared__ int s_pre[];  // [L * kUnits + 1]
     pdl_wait();
     pdl_trigger();
     const T* __restrict__ x = static_cast<const T*>(a.x);
     const T* __restrict__ dz = static_cast<const T*>(a.dz);
     long long rows = *a.count;
     rows = rows < 0 ? 0 : (rows > a.capacity ? a.capacity : rows);
-    const int item = blockIdx.x;
-    const int split = item / a.T;
-    const int tile = item - split * a.T;
-    const int tm = tile / a.n_tiles, tn = tile - tm * a.n_tiles;
-    const long long rps = ((rows + a.splits - 1) / a.splits + kBKs - 1) / kBKs * kBKs;
-    const long long r_begin = (long long)split * rps;
-    long long r_end = r_begin + rps;
-    if (r_end > rows) r_end = rows;
-    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    const int mm = t & (kTile - 1);
-    const int m = tm * kTile + mm;
-    const bool m_ok = m < a.K;
-    const int l = m_ok ? m / a.C_in : 0, c = m - l * a.C_in;
-    const int o = tn * kTile + mm;
-    const bool o_ok = o < a.C_out;
-    unsigned err = 0;
-    float acc[8][8];
+    unit_positions(a.unit_cnt, a.L * kUnits, s_pre, red);
+    __syncthreads();
+    const int g = blockIdx.x;
+    const int ct = (int)blockIdx.y % a.c_tiles, ot = (int)blockIdx.y / a.c_tiles;
+    const Run run(s_pre, a.L, a.G, g);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (g == 0 && blockIdx.y == 0 && t <= a.L + 1) {
+        const int T_ = s_pre[a.L * kUnits];
+        a.slot_pos[t] = t <= a.L ? s_pre[t * kUnits]
+                                 : ((T_ + a.G - 1) / a.G + kBK - 1) / kBK * kBK;
+    }
+    const long long urows = unit_rows(rows);
+    const int tx = t & 15, ty = t >> 4;  // outputs: c = ty * 4 .., o = tx * 4 .. and 64 + tx * 4 ..
+    // loads: x channel t % 64 of taps t / 64 + 4 i; dz channel t % 128 of taps t / 128 + 2 i
+    const int c = ct * kSimtBC + (t & 63), o = ot * kTile + (t & 127);
+    const bool c_ok = c < a.C_in, o_ok = o < a.C_out;
+    int l = 0;
+    for (long long pos = run.p0; pos < run.p1;) {
+        const long long end = run.segment(pos, l);
+        float acc[4][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
-    for (long long n0 = r_begin; n0 < r_end; n0 += kBKs) {
-#pragma unroll
-        for (int i = 0; i < kBKs / 2; ++i) {
-            const int r = (t >> 7) + 2 * i;
-            const long long n = n0 + r;
-            float av = 0.f, bv = 0.f;
-            if (n < r_end) {
-                if (m_ok) {
-                    const int j = __ldg(a.rb + (long long)l * a.capacity + n);
-                    if (j >= 0 && j < a.x_rows)
-                        av = to_f(x[(long long)j * a.C_in + c]);
-                    else if (j != -1)
-                        err |= kErrIndex;
-                }
-                if (o_ok) bv = to_f(dz[n * a.C_out + o]);
+            for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
+        for (; pos < end; pos += kSimtBatch) {
+            const int want = end - pos < kSimtBatch ? (int)(end - pos) : kSimtBatch;
+            if (t < want) {
+                const int2 e = __ldg(a.unit_list + run.entry(l, (int)pos + t, urows, a.capacity));
+                s_j[t] = e.x - 1;
+                s_n[t] = e.y - 1;
             }
-            As[r][mm] = av;
-            Bs[r][mm] = bv;
+            __syncthreads();
+            float xv[4], zv[8];
+            auto fetch = [&](int k0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k = k0 + (t >> 6) + 4 * i;
+                    const int j = k < want ? s_j[k] : -1;
+                    xv[i] = j >= 0 && c_ok ? to_f(x[(long long)j * a.C_in + c]) : 0.f;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int k = k0 + (t >> 7) + 2 * i;
+                    const int n = k < want ? s_n[k] : -1;
+                    zv[i] = n >= 0 && o_ok ? to_f(dz[(long long)n * a.C_out + o]) : 0.f;
+                }
+            };
+            fetch(0);
+            int buf = 0;
+            for (int k0 = 0; k0 < want; k0 += kSimtBK, buf ^= 1) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) Xs[buf][(t >> 6) + 4 * i][t & 63] = xv[i];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) Zs[buf][(t >> 7) + 2 * i][t & 127] = zv[i];
+                __syncthreads();
+                if (k0 + kSimtBK < want) fetch(k0 + kSimtBK);
+#pragma unroll
+                for (int k = 0; k < kSimtBK; ++k) {
+                    const float4 xa = *reinterpret_cast<const float4*>(&Xs[buf][k][ty * 4]);
+                    const float4 za = *reinterpret_cast<const float4*>(&Zs[buf][k][tx * 4]);
+                    const float4 zb = *reinterpret_cast<const float4*>(&Zs[buf][k][64 + tx * 4]);
+                    const float av[4] = {xa.x, xa.y, xa.z, xa.w};
+                    const float bv[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = fmaf(av[i], bv[jj], acc[i][jj]);
+                }
+            }
+            __syncthreads();  // the list and the buffers are free
         }
-        __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < kBKs; ++k) {
-            float avv[8], bvv[8];
+        float* dst = a.part + ((long long)blockIdx.y * (a.G + a.L) + g + l) * (kSimtBC * kTile);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) avv[i] = As[k][ty * 8 + i];
-#pragma unroll
-            for (int jj = 0; jj < 8; ++jj) bvv[jj] = Bs[k][tx * 8 + jj];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) acc[i][jj] = fmaf(avv[i], bvv[jj], acc[i][jj]);
+        for (int i = 0; i < 4; ++i) {
+            float* d = dst + (ty * 4 + i) * kTile + tx * 4;
+            *reinterpret_cast<float4*>(d) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            *reinterpret_cast<float4*>(d + 64) =
+                make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
         }
-        __syncthreads();
+        pos = end;
+    }
+}
+
+// Lists of the taps of each slot (e and its n) for dgrad.
+struct SlotArgs {
+    const int32_t* row_ptr;
+    const int32_t* taps;
+    int x_rows, L, blocks;
+    long long capL;
+    const int32_t* hist;   // [blocks][L]
+    int32_t* slot_off;     // [L + 1]: where each slot's list starts
+    int32_t* list_n;       // source row of dz, -1: zeros
+    int32_t* list_e;       // row of P
+    unsigned* status;
+};
+
+// Block b of a.blocks: the b-th piece of the mapping, each slot's taps behind
+// those of the pieces before (their counts come with the dz launch).
+__device__ void tap_slots(const SlotArgs& a, int b) {
+    __shared__ int s_tot[HC_MAX_SPIRAL], s_bef[HC_MAX_SPIRAL], s_cur[HC_MAX_SPIRAL];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const long long T = total_taps(a.row_ptr, a.x_rows, a.capL);
+    const long long E = (T + a.blocks - 1) / a.blocks;
+    const long long e0 = b * E, e1 = e0 + E < T ? e0 + E : T;
+    int key0 = e0 + t < e1 ? __ldg(a.taps + e0 + t) : 0;
+    for (int l = warp; l < a.L; l += 8) {
+        int tot = 0, bef = 0;
+        for (int i0 = lane; i0 < a.blocks; i0 += 256) {
+            int h[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                h[q] = i0 + 32 * q < a.blocks ? __ldg(a.hist + (i0 + 32 * q) * a.L + l) : 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                tot += h[q];
+                bef += i0 + 32 * q < b ? h[q] : 0;
+            }
+        }
+        tot = __reduce_add_sync(0xffffffffu, tot);
+        bef = __reduce_add_sync(0xffffffffu, bef);
+        if (lane == 0) {
+            s_tot[l] = tot;
+            s_bef[l] = bef;
+        }
+    }
+    __syncthreads();
+    if (t == 0) {
+        int run = 0;
+        for (int l = 0; l < a.L; ++l) {
+            s_cur[l] = run + s_bef[l];
+            if (b == 0) a.slot_off[l] = run;
+            run += s_tot[l];
+        }
+        if (b == 0) a.slot_off[a.L] = run;
+    }
+    __syncthreads();
+    unsigned err = 0;
+    for (long long e = e0 + t; e - lane < e1; e += 256) {
+        const bool in = e < e1;
+        const int key = key0;
+        if (e + 256 < e1) key0 = __ldg(a.taps + e + 256);
+        int n = -1;
+        const int l = in ? slot_of(key, a.L, a.capL, n) : -1;
+        if (in && n < 0) err |= kErrIndex;
+        const unsigned same = __match_any_sync(0xffffffffu, l);
+        const int leader = __ffs(same) - 1;
+        int at = 0;
+        if (in && lane == leader) at = atomicAdd(&s_cur[l], __popc(same));
+        at = __shfl_sync(0xffffffffu, at, leader) + __popc(same & ((1u << lane) - 1u));
+        if (in) {
+            a.list_n[at] = n;
+            a.list_e[at] = (int)e;
+        }
     }
     if (err) report(a.status, err);
-    float* dst = a.part + (long long)item * kPartElems;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float4* d4 = reinterpret_cast<float4*>(dst + (ty * 8 + i) * kTile + tx * 8);
-        d4[0] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        d4[1] = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
-    }
 }
 
-// dW[m][o] = sum over splits (in order) of the partial tiles.
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int K, int C_out, int n_tiles,
-                                    int T, int splits, float* __restrict__ dW) {
+// One launch for three short independent jobs (each on its own is a launch of
+// 6 to 9 us that leaves the GPU idle):
+//   blocks 0 ..          tap_slots, when dx is wanted;
+//   the next dw_blocks   dW[m][o] = sum over the runs that hold taps of the
+//                        slot of m, in a fixed order;
+//   the rest             dbias[o] = sum of the dz blocks' column sums (8
+//                        columns a block, 32 lanes of blocks each).
+struct ReduceArgs {
+    const float* part;
+    const int32_t* slot_pos;
+    int L, C_in, C_out, BC, c_tiles, G, dw_blocks;
+    float* dW;
+    const float* bpart;
+    int act_blocks;
+    float* dbias;
+};
+
+__global__ void __launch_bounds__(256)
+    bwd_collect_kernel(const ReduceArgs a, const SlotArgs slots) {
+    __shared__ float red[32][9], s_sum[4][64];
     pdl_wait();
     pdl_trigger();
-    const long long total = (long long)K * C_out;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        int o;
-        const int m = (int)div32(e, C_out, o);
-        const int t = (m >> 7) * n_tiles + (o >> 7);
-        const float* src = part + (long long)t * kPartElems + ((m & 127) << 7) + (o & 127);
+    if ((int)blockIdx.x < slots.blocks) {
+        tap_slots(slots, blockIdx.x);
+        return;
+    }
+    const int block = (int)blockIdx.x - slots.blocks;
+    if (block >= a.dw_blocks) {
+        const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+        const int o = (block - a.dw_blocks) * 8 + tx;
         float s = 0.f;
-        for (int sp = 0; sp < splits; ++sp) s += src[(long long)sp * T * kPartElems];
-        dW[e] = s;
+        if (o < a.C_out)
+            for (int b0 = ty; b0 < a.act_blocks; b0 += 32 * 8) {
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    v[q] = b0 + 32 * q < a.act_blocks
+                               ? __ldg(a.bpart + (long long)(b0 + 32 * q) * a.C_out + o)
+                               : 0.f;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) s += v[q];
+            }
+        red[ty][tx] = s;
+        __syncthreads();
+        if (ty == 0 && o < a.C_out) {
+            float tot = 0.f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) tot += red[i][tx];
+            a.dbias[o] = tot;
+        }
+        return;
+    }
+    // 64 entries of dW per block and step, four threads each: thread k adds
+    // the runs first + k, + 4, ... (slot 0 has the most, all rows' taps)
+    const long long total = (long long)a.L * a.C_in * a.C_out;
+    const int Q = a.slot_pos[a.L + 1];
+    const int ei = threadIdx.x & 63, k = threadIdx.x >> 6;
+    for (long long e0 = block * 64ll; e0 < total; e0 += a.dw_blocks * 64ll) {
+        const long long e = e0 + ei;
+        float s = 0.f;
+        if (e < total) {
+            int o, c;
+            const int m = (int)div32(e, a.C_out, o);
+            const int l = (int)div32(m, a.C_in, c);
+            const int s0 = a.slot_pos[l], s1 = a.slot_pos[l + 1];
+            if (s1 > s0) {
+                const int tile = (o / kTile) * a.c_tiles + c / a.BC;
+                const long long stride = (long long)a.BC * kTile;
+                const float* src = a.part + (long long)tile * (a.G + a.L) * stride +
+                                   (long long)(c % a.BC) * kTile + (o & (kTile - 1)) + l * stride;
+                const int g1 = (s1 - 1) / Q;
+                for (int g = s0 / Q + k; g <= g1; g += 32) {
+                    float v[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) v[q] = g + 4 * q <= g1 ? src[(g + 4 * q) * stride] : 0.f;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) s += v[q];
+                }
+            }
+        }
+        s_sum[k][ei] = s;
+        __syncthreads();
+        if (k == 0 && e < total)
+            a.dW[e] = ((s_sum[0][ei] + s_sum[1][ei]) + s_sum[2][ei]) + s_sum[3][ei];
+        __syncthreads();
     }
 }
 
-// Block-range gather-sum for rows of 16-byte chunks (cpr = C_in / VEC of
-// them). A block takes R consecutive input rows r0 .. r0 + R - 1 (ranges
-// blockIdx.x, + gridDim.x, ...). Their taps are one contiguous slice
-// taps[ptr[r0] .. ptr[r0 + R]) of the transposed mapping, copied to shared
-// memory in one coalesced pass (read from global memory instead when it does
-// not fit or the table is malformed there). The block then writes zero
-// chunks for the rows without taps and sums, for every (row with taps,
-// chunk) item, the P chunks of the row's taps in ascending key order, eight
-// loads in flight per thread. Every load of a round trip is issued by all
-// threads at once: row ranges, keys, then P.
-constexpr int kDgThreads = 256;
-constexpr int kDgMaxRows = 1024;
-constexpr int kDgKeys = 8192;
+// ---------------------------------------------------------------- dgrad
+// dx[j] = sum over the taps (n, l) of row j, in (n, l) order, of dz[n] W_l^T.
+// The transposed mapping lists them row by row, so with P[e] = dz[n] W_l^T
+// for its e-th tap every row of dx sums consecutive rows of P. Only the
+// present taps have a row in P (a [rows, L * C_in] product computes, writes
+// and rounds all of them; at 25% density two thirds are absent).
+// tap_slots (above) lists the taps of each slot, so that a tile of the product
+// has one W_l.
+struct TapGemmArgs {
+    const void* dz;
+    const void* W;
+    const int32_t* slot_off;
+    const int32_t* list_n;
+    const int32_t* list_e;
+    void* P;                      // [taps][Cp]
+    int L, C_in, C_out, Cp, c_tiles;
+    unsigned* status;
+};
+
+// Tiles of BM listed taps, slot by slot: s_tile[l] = tiles before slot l. By
+// one warp; s_off[l] = the slot's first list entry.
+template <int BM>
+__device__ __forceinline__ void slot_tiles(const int32_t* slot_off, int L, int* s_off,
+                                           int* s_tile) {
+    const int lane = threadIdx.x & 31;
+    const int off = lane < L ? __ldg(slot_off + lane) : 0;
+    const int nxt = lane < L ? __ldg(slot_off + lane + 1) : 0;
+    const int tiles = (nxt - off + BM - 1) / BM;
+    int x = tiles;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane < L) {
+        s_off[lane] = off;
+        s_tile[lane] = x - tiles;
+    }
+    if (lane == L - 1) {
+        s_off[L] = nxt;
+        s_tile[L] = x;
+    }
+}
+
+// tcgen05: 128 listed taps x BN channels of W_l per item, contraction over
+// C_out. A: the taps' rows of dz, gathered by cp.async as in the forward
+// conv (K-major); B: rows l * C_in + c of W as they lie (K-major, C_out
+// contiguous), by TMA, so no transposed copy of W is needed; both 128-byte
+// swizzled. Each item is short (C_out / 64 stages), so what bounds it is the
+// rows' gather and the scattered rows of P (whole 64-byte pieces). Warps 0-3
+// gather (list entries two items ahead in registers), 9 loads W, 8 issues the
+// MMAs, 4-7 and 10-13 round and store the item before (half of its columns
+// each: with four warps the stores took longer than the gather), two
+// accumulators in turn.
+// With seg_sum, against the product over all (row, slot) pairs and a scattered
+// sum: 114 + 107 -> 48 + 40 us at 167k rows, 9 slots, 128 -> 128, 25% present;
+// 17 + 17 -> 17 + 18 us at 16.4k rows, 12 slots, 64 -> 128, 84% present; fp32,
+// 25k rows, 24% present: 142 + 24 -> 38 + 13 us.
+template <int BN>
+struct TapCfg {
+    static constexpr int kABytes = 128 * 128;
+    static constexpr int kStageBytes = kABytes + BN * 128;
+    static constexpr int kStages = BN == 64 ? 8 : 6;
+    static constexpr uint32_t kTmemCols = 2 * BN;
+    static constexpr int kBars = 2 * kStages + 5;
+    static constexpr int kMisc = kStages * kStageBytes;
+    static constexpr int kEpi = kMisc + (8 * kBars + 16 + 2 * 33 * 4 + 127) / 128 * 128;
+    static constexpr size_t kSmem = 1024 + kEpi + 8 * 2048;
+    // D fp32, A and B bf16, both K-major, N = BN, M = 128
+    static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
+                                       ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+};
+
+constexpr int kTapEpilogueWarps = 8;  // 4-7 and 10-13: half of the columns each
+constexpr int kTapThreads = (kIndexWarp + 1 + 4) * 32;
+
+template <int BN>
+__global__ void __launch_bounds__(kTapThreads, 1)
+    tap_gemm_tc_kernel(const TapGemmArgs a, const __grid_constant__ CUtensorMap tmap_w) {
+    using C = TapCfg<BN>;
+    constexpr int kStages = C::kStages;
+    constexpr int kWeightWarp = kIndexWarp;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* const base_ptr = smem_raw + (base - raw);
+    const uint32_t sBar = base + C::kMisc;
+    auto full_bar = [&](int s) { return sBar + 8u * s; };
+    auto empty_bar = [&](int s) { return sBar + 8u * (kStages + s); };
+    auto tfull_bar = [&](int i) { return sBar + 8u * (2 * kStages + i); };
+    auto tempty_bar = [&](int i) { return sBar + 8u * (2 * kStages + 2 + i); };
+    const uint32_t fin_bar = sBar + 8u * (2 * kStages + 4);
+    uint8_t* const misc = base_ptr + C::kMisc + 8 * C::kBars;
+    volatile uint32_t* const tmem_holder = reinterpret_cast<volatile uint32_t*>(misc);
+    volatile int* const abort_flag = reinterpret_cast<volatile int*>(misc + 4);
+    int* const s_off = reinterpret_cast<int*>(misc + 16);
+    int* const s_tile = s_off + 33;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(full_bar(s), kProducerWarps * 32 + 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(tfull_bar(i), 1);
+            mbar_init(tempty_bar(i), kTapEpilogueWarps * 32);
+        }
+        mbar_init(fin_bar, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == kWeightWarp && lane == 0) prefetch_tensormap(&tmap_w);
+    if (warp == kMmaWarp) {
+        tmem_alloc(smem_u32((const void*)tmem_holder), C::kTmemCols);
+        tmem_relinquish();
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (warp == 0) slot_tiles<128>(a.slot_off, a.L, s_off, s_tile);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+    const long long items = (long long)s_tile[a.L] * a.c_tiles;
+    const int nkb = (a.C_out + 63) / 64;
+    // item w: tile w / c_tiles (slot l, list entries [first, first + 128) of
+    // the slot's), channels c0 ..
+    auto locate = [&](long long w, int& l, int& first, int& c0) {
+        const int tile = (int)(w / a.c_tiles);
+        c0 = (int)(w - (long long)tile * a.c_tiles) * BN;
+        while (s_tile[l + 1] <= tile) ++l;
+        first = s_off[l] + (tile - s_tile[l]) * 128;
+    };
+
+    if (warp < kProducerWarps) {
+        const __nv_bfloat16* __restrict__ dz = static_cast<const __nv_bfloat16*>(a.dz);
+        const int t = threadIdx.x, q = t & 7;
+        int n1[8], n2[8];  // list entries of the next item and the one after it
+        int l = 0;
+        auto entries = [&](long long w, int (&n)[8]) {
+            int first, c0;
+            if (w < items) {
+                locate(w, l, first, c0);
+                const int end = s_off[l + 1];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int e = first + (t >> 3) + 16 * i;
+                    n[i] = e < end ? __ldg(a.list_n + e) : -1;
+                }
+            }
+        };
+        entries(blockIdx.x, n1);
+        entries(blockIdx.x + (long long)gridDim.x, n2);
+        int st = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (long long w = blockIdx.x; w < items && ok; w += gridDim.x) {
+            int n[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                n[i] = n1[i];
+                n1[i] = n2[i];
+            }
+            entries(w + 2ll * gridDim.x, n2);
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(empty_bar(st), ph ^ 1u, abort_flag, a.status)) {
+                    ok = false;
+                    break;
+                }
+                const int k = kb * 64 + q * 8;
+                const uint32_t a_st = base + st * C::kStageBytes;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = (t >> 3) + 16 * i;
+                    const bool v = n[i] >= 0 && k < a.C_out;
+                    cp_async_16(a_st + r * 128 + ((q ^ (r & 7)) << 4),
+                                dz + (v ? (long long)n[i] * a.C_out + k : 0), v);
+                }
+                cp_async_arrive_noinc(full_bar(st));
+                if (++st == kStages) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+            }
+        }
+        cp_async_wait_all();
+    } else if (warp == kWeightWarp) {
+        if (lane == 0) {
+            long long it = 0;
+            int st = 0, l = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long w = blockIdx.x; w < items && ok; w += gridDim.x) {
+                int first, c0;
+                locate(w, l, first, c0);
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!mbar_wait(empty_bar(st), ph ^ 1u, abort_flag, a.status)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_arrive_expect_tx(full_bar(st), BN * 128);
+                    tma_load_2d(base + st * C::kStageBytes + C::kABytes, &tmap_w, kb * 64,
+                                l * a.C_in + c0, full_bar(st));
+                    ++it;
+                    if (++st == kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            if (!ok)  // copies already issued land before the CTA exits
+                for (long long j = it > kStages ? it - kStages : 0; j < it; ++j)
+                    mbar_wait_drain(full_bar((int)(j % kStages)), (uint32_t)((j / kStages) & 1),
+                                    a.status);
+        }
+        __syncwarp();
+    } else if (warp == kMmaWarp) {
+        if (lane == 0) {
+            int st = 0, lt = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long w = blockIdx.x; w < items && ok; w += gridDim.x, ++lt) {
+                const int acc = lt & 1;
+                if (!mbar_wait(tempty_bar(acc), (uint32_t)(((lt >> 1) & 1) ^ 1), abort_flag,
+                               a.status))
+                    break;
+                tc_fence_after();
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!mbar_wait(full_bar(st), ph, abort_flag, a.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    fence_proxy_async_smem();
+                    const uint32_t a_st = base + st * C::kStageBytes, b_st = a_st + C::kABytes;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        tc_mma_bf16(tmem_base + (uint32_t)(acc * BN),
+                                    desc_sw128(a_st + k * 32, 16, 1024),
+                                    desc_sw128(b_st + k * 32, 16, 1024), C::kIdesc,
+                                    (kb | k) != 0 ? 1u : 0u);
+                    tc_commit(empty_bar(st));
+                    if (++st == kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                tc_commit(tfull_bar(acc));
+            }
+            tc_commit(fin_bar);
+            mbar_wait_drain(fin_bar, 0, a.status);
+        }
+        __syncwarp();
+    } else {
+        // lane = listed tap; its 32-column pieces leave through a 2 KB buffer
+        // as in the forward conv: a store writes eight taps x 64 bytes
+        const int ew = warp & 3;                       // TMEM lanes 32 ew ..
+        const int half = warp < kMmaWarp ? 0 : 1;      // columns half * BN / 2 ..
+        const uint32_t stage = base + C::kEpi + (half * 4 + (warp < kMmaWarp ? ew : warp - 10)) * 2048;
+        __nv_bfloat16* P = static_cast<__nv_bfloat16*>(a.P);
+        int lt = 0, l = 0, c0 = 0, c0_next = 0;
+        long long e_next = -1;  // the next item's, read one item ahead
+        auto entry = [&](long long w) {
+            if (w >= items) return;
+            int first;
+            locate(w, l, first, c0_next);
+            const int i = first + ew * 32 + lane;
+            e_next = i < s_off[l + 1] ? __ldg(a.list_e + i) : -1;
+        };
+        entry(blockIdx.x);
+        for (long long w = blockIdx.x; w < items; w += gridDim.x, ++lt) {
+            const long long e = e_next;
+            c0 = c0_next;
+            entry(w + gridDim.x);
+            const int acc = lt & 1;
+            long long ek[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ek[k] = __shfl_sync(0xffffffffu, e, 8 * k + (lane >> 2));
+            if (!mbar_wait(tfull_bar(acc), (uint32_t)((lt >> 1) & 1), abort_flag, a.status)) break;
+            tc_fence_after();
+#pragma unroll 1
+            for (int cb = half * (BN / 64); cb < (half + 1) * (BN / 64); ++cb) {
+                uint32_t r[32];
+                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(ew * 32) << 16) +
+                                       (uint32_t)(acc * BN + cb * 32),
+                                   r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int j8 = 0; j8 < 4; ++j8) {
+                    uint32_t p[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const __nv_bfloat162 v =
+                            __floats2bfloat162_rn(__uint_as_float(r[8 * j8 + 2 * h]),
+                                                  __uint_as_float(r[8 * j8 + 2 * h + 1]));
+                        p[h] = *reinterpret_cast<const uint32_t*>(&v);
+                    }
+                    sts_v4(stage + (uint32_t)(lane * 64 + ((j8 ^ ((lane >> 1) & 3)) << 4)),
+                           make_uint4(p[0], p[1], p[2], p[3]));
+                }
+                __syncwarp();
+                const int col = c0 + cb * 32 + (lane & 3) * 8;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int R = 8 * k + (lane >> 2);
+                    const uint4 v =
+                        lds_u4(stage + (uint32_t)(R * 64 + (((lane & 3) ^ ((R >> 1) & 3)) << 4)));
+                    if (col < a.Cp && ek[k] >= 0)
+                        *reinterpret_cast<uint4*>(P + ek[k] * a.Cp + col) = v;
+                }
+                __syncwarp();
+            }
+            tc_fence_before();
+            mbar_arrive(tempty_bar(acc));
+        }
+    }
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, C::kTmemCols);
+    }
+}
+
+// CUDA cores: 64 listed taps x 64 channels per item, 4 x 4 per thread over
+// chunks of 32 of C_out (both operands' rows are contiguous along it and
+// are turned round on their way into shared memory).
+constexpr int kTgBM = 64, kTgBN = 64, kTgBK = 32;
 
 template <typename T>
-__global__ void __launch_bounds__(kDgThreads, 4)
-    dgrad_range_kernel(const T* __restrict__ P, const int32_t* __restrict__ ptr,
-                       const int32_t* __restrict__ taps, int x_rows, int R, int C_in,
-                       long long capL, T* __restrict__ dx, unsigned* status) {
-    constexpr int VEC = 16 / sizeof(T);
-    __shared__ int32_t s_ptr[kDgMaxRows + 1];
-    __shared__ uint16_t s_busy[kDgMaxRows];
-    __shared__ uint8_t s_on[kDgMaxRows];
-    __shared__ int32_t s_keys[kDgKeys];
+__global__ void __launch_bounds__(256) tap_gemm_simt_kernel(const TapGemmArgs a) {
+    __shared__ __align__(16) float As[kTgBK][kTgBM + 4];
+    __shared__ __align__(16) float Bs[kTgBK][kTgBN + 4];
+    __shared__ int s_off[33], s_tile[33], s_e[kTgBM];
+    pdl_wait();
+    pdl_trigger();
+    if (threadIdx.x < 32) slot_tiles<kTgBM>(a.slot_off, a.L, s_off, s_tile);
+    __syncthreads();
+    const T* __restrict__ dz = static_cast<const T*>(a.dz);
+    const T* __restrict__ W = static_cast<const T*>(a.W);
+    T* __restrict__ P = static_cast<T*>(a.P);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    const int kk = t & 31, row = t >> 5;  // loads: k = kk, rows row + 8 i
+    const long long items = (long long)s_tile[a.L] * a.c_tiles;
+    int l = 0;
+    for (long long w = blockIdx.x; w < items; w += gridDim.x) {
+        const int tile = (int)(w / a.c_tiles);
+        const int c0 = (int)(w - (long long)tile * a.c_tiles) * kTgBN;
+        while (s_tile[l + 1] <= tile) ++l;
+        const int first = s_off[l] + (tile - s_tile[l]) * kTgBM, end = s_off[l + 1];
+        if (t < kTgBM) s_e[t] = first + t < end ? __ldg(a.list_e + first + t) : -1;
+        int n[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = first + row + 8 * i;
+            n[i] = e < end ? __ldg(a.list_n + e) : -1;
+        }
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        float av[8], bv[8];
+        auto fetch = [&](int k0) {
+            const int k = k0 + kk;
+            const bool in = k < a.C_out;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                av[i] = in && n[i] >= 0 ? to_f(dz[(long long)n[i] * a.C_out + k]) : 0.f;
+                const int c = c0 + row + 8 * i;
+                bv[i] = in && c < a.C_in ? to_f(W[((long long)l * a.C_in + c) * a.C_out + k]) : 0.f;
+            }
+        };
+        fetch(0);
+        for (int k0 = 0; k0 < a.C_out; k0 += kTgBK) {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                As[kk][row + 8 * i] = av[i];
+                Bs[kk][row + 8 * i] = bv[i];
+            }
+            __syncthreads();
+            if (k0 + kTgBK < a.C_out) fetch(k0 + kTgBK);
+#pragma unroll
+            for (int k = 0; k < kTgBK; ++k) {
+                const float4 x4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
+                const float4 w4 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
+                const float xr[4] = {x4.x, x4.y, x4.z, x4.w}, wr[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xr[i], wr[j], acc[i][j]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const long long e = s_e[ty * 4 + i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = c0 + tx * 4 + j;
+                if (e >= 0 && c < a.Cp) P[e * a.Cp + c] = from_f<T>(acc[i][j]);
+            }
+        }
+        __syncthreads();  // s_e is free
+    }
+}
+
+// dx[j] = sum of P[ptr[j]] .. P[ptr[j + 1] - 1]. A block takes R consecutive
+// rows, their table in shared memory. Most rows of a dense input have no tap:
+// those with taps are listed first, so that every thread of the block then has
+// a (row, 16-byte chunk) item to sum, four taps in flight, and the others are
+// zeroed by stores in order. (With the items dealt out row by row, empty rows
+// included, the few long rows of a warp ran one after the other: 79 us at 335k
+// rows, 5% of them with taps.) Short ranges, one block each: a compact input's
+// active rows are its first ones, so with longer ranges (R = 1024) a quarter
+// of the blocks had all the work at 25% density (103 us instead of 40). A
+// row whose range leaves the table is reported and becomes zeros.
+constexpr int kSegRows = 128;
+
+template <typename T>
+__global__ void __launch_bounds__(256, 6)
+    seg_sum_kernel(const T* __restrict__ P, const int32_t* __restrict__ ptr, int x_rows, int C_in,
+                   int Cp, long long capL, T* __restrict__ dx, int vec_ok, unsigned* status) {
+    constexpr int VEC = 16 / (int)sizeof(T);
+    __shared__ int32_t s_ptr[kSegRows + 1];
+    __shared__ uint16_t s_busy[kSegRows];
+    __shared__ uint8_t s_on[kSegRows];
     __shared__ int s_nb;
     pdl_wait();
     pdl_trigger();
     const int t = threadIdx.x, lane = t & 31;
-    const int cpr = C_in / VEC;
-    for (long long r0 = (long long)blockIdx.x * R; r0 < x_rows; r0 += (long long)gridDim.x * R) {
-        const int n = x_rows - r0 < R ? (int)(x_rows - r0) : R;
-        for (int i = t; i <= n; i += kDgThreads) s_ptr[i] = __ldg(ptr + r0 + i);
-        if (t == 0) s_nb = 0;
-        __syncthreads();
-        const int base = s_ptr[0], top = s_ptr[n];
-        const bool in_smem = base >= 0 && top >= base && top - base <= kDgKeys && top <= capL;
-        // the key slice, while the rows with taps are listed
-        if (in_smem)
-            for (int i = t; i < top - base; i += kDgThreads) s_keys[i] = __ldg(taps + base + i);
-        for (int i0 = 0; i0 < n; i0 += kDgThreads) {
-            const int i = i0 + t;
-            bool on = false;
-            if (i < n) {
-                const int a = s_ptr[i], b = s_ptr[i + 1];
-                const bool ok = a >= 0 && b >= a && b <= capL && (!in_smem || (a >= base && b <= top));
-                if (!ok) report(status, kErrIndex);
-                on = ok && b > a;
-                s_on[i] = on ? 1 : 0;
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, on);
-            int wbase = 0;
-            if (lane == 0 && bal) wbase = atomicAdd(&s_nb, __popc(bal));
-            wbase = __shfl_sync(0xffffffffu, wbase, 0);
-            if (on) s_busy[wbase + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
-        }
-        __syncthreads();
-        // rows without taps: zeros, consecutive chunks per thread
-        for (int f = t; f < n * cpr; f += kDgThreads) {
-            int c;
-            const int i = (int)div32(f, cpr, c);
-            if (!s_on[i])
-                *reinterpret_cast<uint4*>(dx + (r0 + i) * C_in + c * VEC) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        // rows with taps
-        const int nb = s_nb;
-        const int32_t* kp = in_smem ? s_keys : taps;
-        const int koff = in_smem ? base : 0;
-        for (int f = t; f < nb * cpr; f += kDgThreads) {
-            int c;
-            const int bi = (int)div32(f, cpr, c);
-            const int i = s_busy[bi];
-            const int a = s_ptr[i] - koff, b = s_ptr[i + 1] - koff;
-            float acc[VEC];
-#pragma unroll
-            for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
-            for (int e0 = a; e0 < b; e0 += 8) {
-                uint4 raw[8];
-                bool use[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int key = e0 + q < b ? kp[e0 + q] : -1;
-                    use[q] = key >= 0 && (long long)key < capL;
-                    if (e0 + q < b && !use[q]) report(status, kErrIndex);
-                    // key n*L + l: P's row n, slot l starts at (n*L + l)*C_in
-                    if (use[q])
-                        raw[q] = *reinterpret_cast<const uint4*>(P + (long long)key * C_in + c * VEC);
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (!use[q]) continue;
-                    const T* v = reinterpret_cast<const T*>(&raw[q]);
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) acc[k] += to_f(v[k]);
-                }
-            }
+    const int cpr = Cp / VEC;
+    const long long r0 = (long long)blockIdx.x * kSegRows;
+    const int n = x_rows - r0 < kSegRows ? (int)(x_rows - r0) : kSegRows;
+    if (t <= n) s_ptr[t] = __ldg(ptr + r0 + t);
+    const long long total = total_taps(ptr, x_rows, capL);
+    if (t == 0) s_nb = 0;
+    __syncthreads();
+    bool on = false;
+    if (t < n) {
+        const int a0 = s_ptr[t], b0 = s_ptr[t + 1];
+        const bool ok = a0 >= 0 && b0 >= a0 && b0 <= total;
+        if (!ok) report(status, kErrIndex);
+        on = ok && b0 > a0;
+        s_on[t] = on ? 1 : 0;
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, on);
+    int at = 0;
+    if (lane == 0 && bal) at = atomicAdd(&s_nb, __popc(bal));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (on) s_busy[at + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)t;
+    __syncthreads();
+    auto store = [&](long long row, int col, const float* v) {
+        T* dst = dx + row * C_in + col;
+        if (vec_ok) {
             uint4 out;
             T* ov = reinterpret_cast<T*>(&out);
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) ov[k] = from_f<T>(acc[k]);
-            *reinterpret_cast<uint4*>(dx + (r0 + i) * C_in + c * VEC) = out;
+            for (int k = 0; k < VEC; ++k) ov[k] = from_f<T>(v[k]);
+            *reinterpret_cast<uint4*>(dst) = out;
+        } else {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k)
+                if (col + k < C_in) dst[k] = from_f<T>(v[k]);
         }
-        __syncthreads();  // the shared tables are reused by the next range
+    };
+    const int nb = s_nb;
+    if (nb < n) {
+        const float zero[VEC] = {};
+        for (int f = t; f < n * cpr; f += 256) {
+            const int i = (unsigned)f / (unsigned)cpr;
+            if (!s_on[i]) store(r0 + i, (f - i * cpr) * VEC, zero);
+        }
+    }
+    for (int f = t; f < nb * cpr; f += 256) {
+        const int bi = (unsigned)f / (unsigned)cpr;
+        const int i = s_busy[bi], col = (f - bi * cpr) * VEC;
+        const int e1 = s_ptr[i + 1];
+        float acc[VEC];
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
+        for (int e = s_ptr[i]; e < e1; e += 4) {
+            uint4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (e + q < e1)
+                    v[q] = __ldg(reinterpret_cast<const uint4*>(P + (long long)(e + q) * Cp + col));
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (e + q < e1) {
+                    const T* p = reinterpret_cast<const T*>(&v[q]);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) acc[k] += to_f(p[k]);
+                }
+        }
+        store(r0 + i, col, acc);
     }
 }
 
+template <typename Kernel>
+hc_status allow_smem(const DeviceCtx* ctx, Kernel k, size_t bytes, bool (&done)[64],
+                     const char* what) {
+    if (done[ctx->device]) return HC_OK;
+    hc_status st = check_cuda(
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
+    if (st == HC_OK) done[ctx->device] = true;
+    return st;
+}
+
+template <int BC>
+hc_status launch_wgrad_tc(const DeviceCtx* ctx, const WgradArgs& w, cudaStream_t s) {
+    static bool done[64] = {};
+    hc_status st = allow_smem(ctx, wgrad_tc_kernel<BC>, WgradCfg<BC>::smem_bytes(HC_MAX_SPIRAL),
+                              done, "cudaFuncSetAttribute(wgrad_tc_kernel)");
+    if (st != HC_OK) return st;
+    return launch_pdl(wgrad_tc_kernel<BC>, dim3((unsigned)w.G, (unsigned)(w.c_tiles * w.o_tiles)),
+                      dim3(kThreadsTc), WgradCfg<BC>::smem_bytes(w.L), s, "wgrad_tc_kernel", w);
+}
+
+template <int BN>
+hc_status launch_tap_gemm_tc(const DeviceCtx* ctx, const TapGemmArgs& g, cudaStream_t s) {
+    static bool done[64] = {};
+    hc_status st = allow_smem(ctx, tap_gemm_tc_kernel<BN>, TapCfg<BN>::kSmem, done,
+                              "cudaFuncSetAttribute(tap_gemm_tc_kernel)");
+    if (st != HC_OK) return st;
+    CUtensorMap tw;
+    st = encode_map_2d(&tw, g.W, (long long)g.L * g.C_in, g.C_out, 64, BN);
+    if (st != HC_OK) return st;
+    return launch_pdl(tap_gemm_tc_kernel<BN>, dim3((unsigned)ctx->num_sms), dim3(kTapThreads),
+                      TapCfg<BN>::kSmem, s, "tap_gemm_tc_kernel", g, tw);
+}
+
 template <typename T>
-hc_status launch_dgrad_typed(const DeviceCtx* ctx, const void* P, const int32_t* ptr,
-                             const int32_t* taps, int x_rows, int L, int C_in, long long capacity,
-                             void* dx, cudaStream_t s) {
-    const uintptr_t al = (uintptr_t)P | (uintptr_t)dx;
-    const int vec16 = 16 / (int)sizeof(T);
-    const bool wide = C_in % vec16 == 0 && al % 16 == 0;
-    const int vec = wide ? vec16 : 1;
-    if (wide && (long long)kDgMaxRows * (C_in / vec16) < (1ll << 31)) {
-        // ranges of R rows, about one per resident block (4 per SM)
-        const long long want = (long long)ctx->num_sms * 4;
-        long long R = ((long long)x_rows + want - 1) / want;
-        R = (R + 31) / 32 * 32;
-        if (R < 256) R = 256;
-        if (R > kDgMaxRows) R = kDgMaxRows;
-        long long blocks = ((long long)x_rows + R - 1) / R;
-        if (blocks > want) blocks = want;
-        if (blocks < 1) blocks = 1;
-        return launch_pdl(dgrad_range_kernel<T>, dim3((unsigned)blocks), dim3(kDgThreads), 0, s,
-                          "dgrad_range_kernel", (const T*)P, ptr, taps, x_rows, (int)R, C_in,
-                          capacity * L, (T*)dx, ctx->status);
-    }
-    long long blocks = ((long long)x_rows * (C_in / vec) + 255) / 256;
-    const long long cap = (long long)ctx->num_sms * 8;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    if (wide)
-        return launch_pdl(dgrad_kernel<T, uint4>, dim3((unsigned)blocks), dim3(256), 0, s,
-                          "dgrad_kernel", (const T*)P, ptr, taps, x_rows, L, C_in, capacity, (T*)dx,
-                          ctx->status);
-    return launch_pdl(dgrad_kernel<T, T>, dim3((unsigned)blocks), dim3(256), 0, s, "dgrad_kernel",
-                      (const T*)P, ptr, taps, x_rows, L, C_in, capacity, (T*)dx, ctx->status);
+hc_status launch_act(const BwdArgs& b, const PrepArgs& prep, bool wide, T* dz, float* bpart,
+                     unsigned* status, cudaStream_t s) {
+    const dim3 grid((unsigned)(prep.act_blocks + prep.unit_blocks + prep.hist_blocks));
+    return launch_pdl(wide ? act_bwd_vec_kernel<T> : act_bwd_kernel<T>, grid, dim3(256), 0, s,
+                      "act_bwd_kernel", (const T*)b.y, (const T*)b.dy, b.count,
+                      (long long)b.capacity, b.C_out, b.act, dz, bpart, prep, status);
 }
 
 }  // namespace
@@ -980,161 +1766,172 @@ hc_status launch_rulebook_transpose(const DeviceCtx* ctx, const int32_t* rb, con
 
 hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s) {
     const bool bf = b.dt == HC_BF16;
-    const int eb = bf ? 2 : 4;
-    const int K = b.L * b.C_in;
-    // Work split of wgrad: 128 x 128 tiles of dW, rows split to fill the SMs.
-    const int m_tiles = (K + kTile - 1) / kTile, n_tiles = (b.C_out + kTile - 1) / kTile;
-    const int T = m_tiles * n_tiles;
-    int splits = 1;
-    {
-        long long max_splits = ((long long)b.capacity + kBK - 1) / kBK;
-        const long long cap_splits = 8ll * ctx->num_sms / T + 1;
-        if (max_splits > cap_splits) max_splits = cap_splits;
-        if (max_splits < 1) max_splits = 1;
-        double best = 0.0;
-        for (int sp = 1; sp <= max_splits; ++sp) {
-            const long long items = (long long)sp * T;
-            const long long waves = (items + ctx->num_sms - 1) / ctx->num_sms;
-            const double eff = (double)items / (double)(waves * ctx->num_sms);
-            if (eff > best + 1e-9) {
-                best = eff;
-                splits = sp;
-            }
-            if (eff >= 0.95) break;
-        }
-    }
-    const long long items = (long long)splits * T;
+    const int eb = bf ? 2 : 4, vec = 16 / eb;
+    const long long capL = (long long)b.capacity * b.L;
     // dz: 16-byte chunks when a row is a whole number of them dividing 256
-    const int act_vec = 16 / eb, act_cpr = b.C_out / act_vec;
-    const bool act_wide = b.C_out % act_vec == 0 && 256 % act_cpr == 0 &&
+    const int act_cpr = b.C_out / vec;
+    const bool act_wide = b.C_out % vec == 0 && 256 % act_cpr == 0 &&
                           ((uintptr_t)b.y | (uintptr_t)b.dy) % 16 == 0;
     const long long act_rows = act_wide ? kActVecItems / act_cpr : kActRowsPerBlock;
-    long long act_blocks_ll = ((long long)b.capacity + act_rows - 1) / act_rows;
+    long long act_blocks = ((long long)b.capacity + act_rows - 1) / act_rows;
     const long long act_cap = (act_wide ? 4ll : 8ll) * ctx->num_sms;
-    if (act_blocks_ll > act_cap) act_blocks_ll = act_cap;
-    const int act_blocks = (int)(act_blocks_ll > 0 ? act_blocks_ll : 1);
+    if (act_blocks > act_cap) act_blocks = act_cap;
+    if (act_blocks < 1) act_blocks = 1;
 
-    // workspace: dz | P | W^T | wgrad partials | dbias partials
-    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-    const size_t dz_bytes = up((size_t)b.capacity * b.C_out * eb);
-    const size_t p_bytes = b.dx ? up((size_t)b.capacity * K * eb) : 0;
-    const size_t wt_bytes = b.dx ? up((size_t)K * b.C_out * eb) : 0;
-    const size_t part_bytes = b.dW ? up(sizeof(float) * (size_t)items * kPartElems) : 0;
-    const size_t bp_bytes = up(sizeof(float) * (size_t)(act_blocks > 0 ? act_blocks : 1) * b.C_out);
-    uint8_t* ws = (uint8_t*)stream_workspace(s, dz_bytes + p_bytes + wt_bytes + part_bytes + bp_bytes);
+    // wgrad: tensor cores for bf16 rows of whole 16-byte chunks; one CTA per
+    // SM over all tiles (two on CUDA cores)
+    const bool w_tc = bf && b.C_in % 8 == 0 && b.C_out % 8 == 0 && (uintptr_t)b.x % 16 == 0;
+    const int BC = w_tc && b.C_in > 64 ? 128 : 64;
+    const int c_tiles = (b.C_in + BC - 1) / BC, o_tiles = (b.C_out + kTile - 1) / kTile;
+    int G = (w_tc ? 1 : 2) * ctx->num_sms / (c_tiles * o_tiles);
+    if (G < 1) G = 1;
+    // tap GEMM: P's rows padded to whole 16-byte chunks
+    const int Cp = (b.C_in + vec - 1) / vec * vec;
+    const bool p_tc = bf && b.C_out % 8 == 0 && (uintptr_t)b.W % 16 == 0;
+
+    const int slot_blocks = 2 * ctx->num_sms;
+
+    // workspace
+    size_t total = 0;
+    auto take = [&](bool wanted, size_t bytes) {
+        const size_t at = total;
+        if (wanted) total += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t dz_at = take(true, (size_t)b.capacity * b.C_out * eb);
+    const size_t bp_at = take(true, sizeof(float) * (size_t)act_blocks * b.C_out);
+    const size_t part_at = take(b.dW, sizeof(float) * (size_t)c_tiles * o_tiles * (G + b.L) * BC * kTile);
+    const size_t unit_at = take(b.dW, sizeof(int32_t) * (size_t)b.L * kUnits);
+    const size_t ul_at = take(b.dW, sizeof(int2) * (size_t)capL);
+    const size_t pos_at = take(b.dW, sizeof(int32_t) * (size_t)(b.L + 2));
+    const size_t p_at = take(b.dx, (size_t)capL * Cp * eb);
+    const size_t ln_at = take(b.dx, sizeof(int32_t) * (size_t)capL);
+    const size_t le_at = take(b.dx, sizeof(int32_t) * (size_t)capL);
+    const size_t hist_at = take(b.dx, sizeof(int32_t) * (size_t)slot_blocks * b.L);
+    const size_t off_at = take(b.dx, sizeof(int32_t) * (size_t)(b.L + 1));
+    uint8_t* ws = (uint8_t*)stream_workspace(s, total);
     if (!ws) return HC_ERR_CUDA;
-    void* dz = ws;
-    void* P = ws + dz_bytes;
-    void* Wt = ws + dz_bytes + p_bytes;
-    float* part = (float*)(ws + dz_bytes + p_bytes + wt_bytes);
-    float* bpart = (float*)(ws + dz_bytes + p_bytes + wt_bytes + part_bytes);
+    void* dz = ws + dz_at;
+    float* bpart = (float*)(ws + bp_at);
 
-    hc_status st;
-    if (act_wide && bf)
-        st = launch_pdl(act_bwd_vec_kernel<__nv_bfloat16>, dim3((unsigned)act_blocks), dim3(256), 0,
-                        s, "act_bwd_vec_kernel", (const __nv_bfloat16*)b.y,
-                        (const __nv_bfloat16*)b.dy, b.count, (long long)b.capacity, b.C_out, b.act,
-                        (__nv_bfloat16*)dz, bpart, ctx->status);
-    else if (act_wide)
-        st = launch_pdl(act_bwd_vec_kernel<float>, dim3((unsigned)act_blocks), dim3(256), 0, s,
-                        "act_bwd_vec_kernel", (const float*)b.y, (const float*)b.dy, b.count,
-                        (long long)b.capacity, b.C_out, b.act, (float*)dz, bpart, ctx->status);
-    else if (bf)
-        st = launch_pdl(act_bwd_kernel<__nv_bfloat16>, dim3((unsigned)act_blocks), dim3(256), 0, s,
-                        "act_bwd_kernel", (const __nv_bfloat16*)b.y, (const __nv_bfloat16*)b.dy,
-                        b.count, (long long)b.capacity, b.C_out, b.act, (__nv_bfloat16*)dz, bpart,
-                        ctx->status);
-    else
-        st = launch_pdl(act_bwd_kernel<float>, dim3((unsigned)act_blocks), dim3(256), 0, s,
-                        "act_bwd_kernel", (const float*)b.y, (const float*)b.dy, b.count,
-                        (long long)b.capacity, b.C_out, b.act, (float*)dz, bpart, ctx->status);
+    PrepArgs prep{};
+    prep.act_blocks = (int)act_blocks;
+    prep.unit_blocks = b.dW ? (b.L * kUnits + 7) / 8 : 0;
+    prep.hist_blocks = b.dx ? slot_blocks : 0;
+    prep.rb = b.rulebook;
+    prep.L = b.L;
+    prep.x_rows = b.x_rows;
+    prep.unit_cnt = (int32_t*)(ws + unit_at);
+    prep.unit_list = (int2*)(ws + ul_at);
+    prep.status = ctx->status;
+    prep.row_ptr = b.row_ptr;
+    prep.taps = b.taps;
+    prep.hist = (int32_t*)(ws + hist_at);
+    hc_status st = bf ? launch_act<__nv_bfloat16>(b, prep, act_wide, (__nv_bfloat16*)dz, bpart,
+                                                  ctx->status, s)
+                      : launch_act<float>(b, prep, act_wide, (float*)dz, bpart, ctx->status, s);
     if (st != HC_OK) return st;
-    if (b.dbias) {
-        st = launch_pdl(dbias_kernel, dim3((unsigned)((b.C_out + 31) / 32)), dim3(32, 32), 0, s,
-                        "dbias_kernel", (const float*)bpart, act_blocks, b.C_out, b.dbias);
-        if (st != HC_OK) return st;
-    }
 
     if (b.dW) {
         WgradArgs w{};
         w.x = b.x;
-        w.rb = b.rulebook;
         w.count = b.count;
         w.dz = dz;
         w.capacity = b.capacity;
-        w.x_rows = b.x_rows;
         w.L = b.L;
         w.C_in = b.C_in;
         w.C_out = b.C_out;
-        w.K = K;
-        w.m_tiles = m_tiles;
-        w.n_tiles = n_tiles;
-        w.T = T;
-        w.splits = splits;
-        w.part = part;
+        w.c_tiles = c_tiles;
+        w.o_tiles = o_tiles;
+        w.G = G;
+        w.unit_cnt = prep.unit_cnt;
+        w.unit_list = prep.unit_list;
+        w.slot_pos = (int32_t*)(ws + pos_at);
+        w.part = (float*)(ws + part_at);
         w.status = ctx->status;
-        const bool tc = bf && b.C_in % 8 == 0 && b.C_out % 8 == 0 && (uintptr_t)b.x % 16 == 0;
-        if (tc) {
-            static bool attr_set[64] = {};
-            if (!attr_set[ctx->device]) {
-                st = check_cuda(cudaFuncSetAttribute(wgrad_tc_kernel,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)kSmemTc),
-                                "cudaFuncSetAttribute(wgrad_tc_kernel)");
-                if (st != HC_OK) return st;
-                attr_set[ctx->device] = true;
-            }
-            st = launch_pdl(wgrad_tc_kernel, dim3((unsigned)items), dim3(kThreadsTc), kSmemTc, s,
-                            "wgrad_tc_kernel", w);
-        } else if (bf) {
-            st = launch_pdl(wgrad_simt_kernel<__nv_bfloat16>, dim3((unsigned)items), dim3(256), 0, s,
-                            "wgrad_simt_kernel", w);
-        } else {
-            st = launch_pdl(wgrad_simt_kernel<float>, dim3((unsigned)items), dim3(256), 0, s,
-                            "wgrad_simt_kernel", w);
-        }
+        const dim3 grid((unsigned)G, (unsigned)(c_tiles * o_tiles));
+        const size_t pre = sizeof(int) * ((size_t)b.L * kUnits + 1);
+        if (w_tc)
+            st = BC == 64 ? launch_wgrad_tc<64>(ctx, w, s) : launch_wgrad_tc<128>(ctx, w, s);
+        else
+            st = launch_pdl(bf ? wgrad_simt_kernel<__nv_bfloat16> : wgrad_simt_kernel<float>, grid,
+                            dim3(256), pre, s, "wgrad_simt_kernel", w);
         if (st != HC_OK) return st;
-        long long rblocks = ((long long)K * b.C_out + 255) / 256;
-        if (rblocks > (long long)ctx->num_sms * 8) rblocks = (long long)ctx->num_sms * 8;
-        st = launch_pdl(wgrad_reduce_kernel, dim3((unsigned)rblocks), dim3(256), 0, s,
-                        "wgrad_reduce_kernel", (const float*)part, K, b.C_out, n_tiles, T, splits,
-                        b.dW);
+    }
+    SlotArgs sl{};
+    if (b.dx) {
+        sl.row_ptr = b.row_ptr;
+        sl.taps = b.taps;
+        sl.x_rows = b.x_rows;
+        sl.L = b.L;
+        sl.blocks = slot_blocks;
+        sl.capL = capL;
+        sl.hist = prep.hist;
+        sl.slot_off = (int32_t*)(ws + off_at);
+        sl.list_n = (int32_t*)(ws + ln_at);
+        sl.list_e = (int32_t*)(ws + le_at);
+        sl.status = ctx->status;
+    }
+    ReduceArgs r{};
+    r.L = b.L;
+    r.C_in = b.C_in;
+    r.C_out = b.C_out;
+    r.BC = BC;
+    r.c_tiles = c_tiles;
+    r.G = G;
+    if (b.dW) {
+        long long blocks = ((long long)b.L * b.C_in * b.C_out + 63) / 64;
+        if (blocks > 8ll * ctx->num_sms) blocks = 8ll * ctx->num_sms;
+        r.dw_blocks = (int)blocks;
+    }
+    r.part = (const float*)(ws + part_at);
+    r.slot_pos = (const int32_t*)(ws + pos_at);
+    r.dW = b.dW;
+    r.bpart = bpart;
+    r.act_blocks = (int)act_blocks;
+    r.dbias = b.dbias;
+    const int collect = sl.blocks + r.dw_blocks + (b.dbias ? (b.C_out + 7) / 8 : 0);
+    if (collect > 0) {
+        st = launch_pdl(bwd_collect_kernel, dim3((unsigned)collect), dim3(256), 0, s,
+                        "bwd_collect_kernel", r, sl);
         if (st != HC_OK) return st;
     }
 
     if (b.dx) {
-        // W^T, then P = dz W^T through the linear conv path, then the gather-sum.
-        const dim3 tg((unsigned)((b.C_out + 31) / 32), (unsigned)((K + 31) / 32)), tb(32, 8);
-        st = bf ? launch_pdl(transpose_kernel<__nv_bfloat16>, tg, tb, 0, s, "transpose_kernel",
-                             (const __nv_bfloat16*)b.W, K, b.C_out, (__nv_bfloat16*)Wt)
-                : launch_pdl(transpose_kernel<float>, tg, tb, 0, s, "transpose_kernel",
-                             (const float*)b.W, K, b.C_out, (float*)Wt);
+        TapGemmArgs g{};
+        g.dz = dz;
+        g.W = b.W;
+        g.slot_off = sl.slot_off;
+        g.list_n = sl.list_n;
+        g.list_e = sl.list_e;
+        g.P = ws + p_at;
+        g.L = b.L;
+        g.C_in = b.C_in;
+        g.C_out = b.C_out;
+        g.Cp = Cp;
+        g.status = ctx->status;
+        if (p_tc) {
+            g.c_tiles = (b.C_in + (b.C_in <= 64 ? 63 : 127)) / (b.C_in <= 64 ? 64 : 128);
+            st = b.C_in <= 64 ? launch_tap_gemm_tc<64>(ctx, g, s) : launch_tap_gemm_tc<128>(ctx, g, s);
+        } else {
+            g.c_tiles = (b.C_in + kTgBN - 1) / kTgBN;
+            st = launch_pdl(bf ? tap_gemm_simt_kernel<__nv_bfloat16> : tap_gemm_simt_kernel<float>,
+                            dim3((unsigned)(4 * ctx->num_sms)), dim3(256), 0, s,
+                            "tap_gemm_simt_kernel", g);
+        }
         if (st != HC_OK) return st;
-        ConvArgs c{};
-        c.x = dz;
-        c.count = b.count;
-        c.W = Wt;
-        c.bias = nullptr;
-        c.y = P;
-        c.capacity = b.capacity;
-        c.x_rows = b.capacity;
-        c.B = 1;
-        c.V = b.capacity;
-        c.L = 1;
-        c.C_in = b.C_out;
-        c.C_out = K;
-        c.K = b.C_out;
-        c.mode = kLinear;
-        c.act = HC_ACT_NONE;
-        st = dispatch_conv(ctx, c, b.dt, s);
-        if (st != HC_OK) return st;
-        st = bf ? launch_dgrad_typed<__nv_bfloat16>(ctx, P, b.row_ptr, b.taps, b.x_rows, b.L, b.C_in,
-                                                    b.capacity, b.dx, s)
-                : launch_dgrad_typed<float>(ctx, P, b.row_ptr, b.taps, b.x_rows, b.L, b.C_in,
-                                            b.capacity, b.dx, s);
-        if (st != HC_OK) return st;
+        const int vec_ok = b.C_in % vec == 0 && (uintptr_t)b.dx % 16 == 0;
+        const long long blocks = ((long long)b.x_rows + kSegRows - 1) / kSegRows;
+        if (bf)
+            st = launch_pdl(seg_sum_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(256), 0, s,
+                            "seg_sum_kernel", (const __nv_bfloat16*)g.P, b.row_ptr, b.x_rows,
+                            b.C_in, Cp, capL, (__nv_bfloat16*)b.dx, vec_ok, ctx->status);
+        else
+            st = launch_pdl(seg_sum_kernel<float>, dim3((unsigned)blocks), dim3(256), 0, s,
+                            "seg_sum_kernel", (const float*)g.P, b.row_ptr, b.x_rows, b.C_in, Cp,
+                            capL, (float*)b.dx, vec_ok, ctx->status);
     }
-    return HC_OK;
+    return st;
 }
 
 }  // namespace hc
