@@ -1,8 +1,8 @@
-// Spiral convolution / linear layer on CUDA cores (FFMA, fp32 accumulate).
-//
-// Used for fp32 (genuine IEEE fp32 multiply-adds: no TF32) and for bf16
-// shapes the tensor-core kernel does not take (channel counts that are not a
-// multiple of 8, e.g. a 45-channel input or a 42- or 1-wide output head).
+// Spiral convolution / linear layer on CUDA cores (FFMA, fp32 accumulate) for
+// bf16 shapes the tensor-core kernel does not take (output channel counts that
+// are not a multiple of 8, misaligned rows), and for the fp32 dense layer at
+// some widths; other fp32 layers have a kernel of their own (conv_f32.cu). And
+// the narrow linear heads of both types.
 //
 // Each CTA owns a 64-row x 64-column output tile and walks K = L*C_in in
 // chunks of KC (128 when K <= 256, else 64): the A chunk is gathered through the per-tile table of source
@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 
 #include "hc_internal.cuh"
+#include "tap_table.cuh"
 
 namespace hc {
 namespace {
@@ -81,66 +82,7 @@ __global__ void __launch_bounds__(kThreads) conv_simt_kernel(const ConvArgs a) {
     for (long long mt = blockIdx.x; mt < m_tiles; mt += gridDim.x) {
         const long long m0 = mt * kBM;
         __syncthreads();  // the previous tile is done with src_tab
-        {
-            // Four threads per row, slots l = part + 4*j: the coordinate, the
-            // spiral entries and the row_of lookups are each issued together
-            // (three dependent round trips per tile).
-            const int r = tid >> 2, part = tid & 3;
-            const long long n = m0 + r;
-            const bool in = n < rows;
-            const long long nn = in ? n : 0;
-            unsigned err = 0;
-            int b = 0, v = 0;
-            if (a.mode == kSparseDenseX || a.mode == kSparseCompactX) {
-                b = __ldg(a.coords + 2 * nn);
-                v = __ldg(a.coords + 2 * nn + 1);
-            } else if (a.mode == kDense) {
-                b = (int)(nn / a.V);
-                v = (int)(nn - (long long)b * a.V);
-            }
-            const bool in_range = b >= 0 && b < a.B && v >= 0 && v < a.V;
-            if (in && !in_range) err |= kErrIndex;
-            const bool ok = in && in_range;
-            if (!ok) b = v = 0;
-            const bool linear = a.mode == kLinear;
-            const bool rb = a.mode == kRulebook;
-            // Loads from clamped, always-valid addresses first; checks after.
-            int u[HC_MAX_SPIRAL / 4];
-#pragma unroll
-            for (int j = 0; j < HC_MAX_SPIRAL / 4; ++j) {
-                const int l = part + 4 * j < L ? part + 4 * j : L - 1;
-                u[j] = linear ? 0
-                       : rb   ? __ldg(a.rulebook + (long long)l * a.capacity + nn)
-                              : __ldg(a.spiral + (long long)v * L + l);
-            }
-#pragma unroll
-            for (int j = 0; j < HC_MAX_SPIRAL / 4; ++j) {
-                const int l = part + 4 * j;
-                if (l >= L) continue;
-                int src = -1;
-                if (ok && linear) {
-                    src = (int)n;
-                } else if (ok && rb) {
-                    if (u[j] < -1 || u[j] >= a.x_rows) err |= kErrIndex;
-                    else src = u[j];
-                } else if (ok) {
-                    const int uu = u[j];
-                    if (uu < -1 || uu >= a.V) err |= kErrIndex;
-                    if (uu >= 0 && uu < a.V) {
-                        const long long dr = (long long)b * a.V + uu;
-                        if (a.mode == kDense) {
-                            src = (int)dr;
-                        } else {
-                            const int jj = __ldg(a.row_of + dr);
-                            if (jj < -1 || jj >= rows) err |= kErrIndex;
-                            if (jj >= 0 && jj < rows) src = a.mode == kSparseDenseX ? (int)dr : jj;
-                        }
-                    }
-                }
-                src_tab[r * L + l] = src;
-            }
-            if (err) report(a.status, err);
-        }
+        fill_tap_table<kBM, kThreads>(a, rows, m0, rows, src_tab, L, 1);
         __syncthreads();
 
         float acc[4][4];
@@ -375,8 +317,10 @@ hc_status launch_head_typed(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_
 // Linear layers on compact rows with few outputs, whose row of x and weights
 // fit in shared memory.
 bool linear_head_supported(const ConvArgs& a, hc_dtype dt) {
-    const int eb = dt == HC_F32 ? 4 : 2;
-    return a.mode == kLinear && a.out_dense == nullptr && a.C_out <= kHeadMaxOut &&
+    // fp32 with more than 16 outputs is faster on the fp32 conv's taller tiles
+    // (64 -> 64 over 4k rows: 12.3 us there, 24.7 us here)
+    const int eb = dt == HC_F32 ? 4 : 2, most = dt == HC_F32 ? 16 : kHeadMaxOut;
+    return a.mode == kLinear && a.out_dense == nullptr && a.C_out <= most &&
            (long long)a.C_in * eb <= kHeadMaxRowBytes &&
            a.C_in * head_wpitch(a.C_out) <= kHeadMaxWFloats;
 }
@@ -386,7 +330,8 @@ hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype d
                         : launch_head_typed<__nv_bfloat16>(ctx, a, s);
 }
 
-hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s) {
+template <typename T>
+static hc_status launch_simt_typed(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
     long long cap_tiles = (a.capacity + kBM - 1) / kBM;
     long long gx = cap_tiles < (long long)ctx->num_sms * 8 ? cap_tiles : (long long)ctx->num_sms * 8;
     if (gx < 1) gx = 1;
@@ -402,27 +347,21 @@ hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt,
                                 "cudaFuncSetAttribute(conv_simt_kernel)");
         };
         const size_t tab_max = sizeof(int) * (size_t)kBM * HC_MAX_SPIRAL;
-        allow(conv_simt_kernel<float, 128>, chunk_smem_bytes<128>() + tab_max);
-        allow(conv_simt_kernel<__nv_bfloat16, 128>, chunk_smem_bytes<128>() + tab_max);
-        allow(conv_simt_kernel<float, 64>, chunk_smem_bytes<64>() + tab_max);
-        allow(conv_simt_kernel<__nv_bfloat16, 64>, chunk_smem_bytes<64>() + tab_max);
+        allow(conv_simt_kernel<T, 128>, chunk_smem_bytes<128>() + tab_max);
+        allow(conv_simt_kernel<T, 64>, chunk_smem_bytes<64>() + tab_max);
         if (st != HC_OK) return st;
         attr_set[ctx->device] = true;
     }
-    if (a.K <= 256) {
-        const size_t smem = chunk_smem_bytes<128>() + tab;
-        if (dt == HC_F32)
-            return launch_pdl(conv_simt_kernel<float, 128>, grid, dim3(kThreads), smem, s,
-                              "conv_simt_kernel", a);
-        return launch_pdl(conv_simt_kernel<__nv_bfloat16, 128>, grid, dim3(kThreads), smem, s,
-                          "conv_simt_kernel", a);
-    }
-    const size_t smem = chunk_smem_bytes<64>() + tab;
-    if (dt == HC_F32)
-        return launch_pdl(conv_simt_kernel<float, 64>, grid, dim3(kThreads), smem, s,
-                          "conv_simt_kernel", a);
-    return launch_pdl(conv_simt_kernel<__nv_bfloat16, 64>, grid, dim3(kThreads), smem, s,
+    if (a.K <= 256)
+        return launch_pdl(conv_simt_kernel<T, 128>, grid, dim3(kThreads),
+                          chunk_smem_bytes<128>() + tab, s, "conv_simt_kernel", a);
+    return launch_pdl(conv_simt_kernel<T, 64>, grid, dim3(kThreads), chunk_smem_bytes<64>() + tab, s,
                       "conv_simt_kernel", a);
+}
+
+hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s) {
+    return dt == HC_F32 ? launch_simt_typed<float>(ctx, a, s)
+                        : launch_simt_typed<__nv_bfloat16>(ctx, a, s);
 }
 
 }  // namespace hc

@@ -114,6 +114,8 @@ struct ConvArgs {
 hc_status launch_compact(const DeviceCtx* ctx, const uint8_t* mask, int B, int V, int32_t* coords,
                          int32_t* row_of, int32_t* offsets, int32_t* count, cudaStream_t s);
 hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
+bool conv_f32_preferred(const ConvArgs& a);
+hc_status launch_conv_f32(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
 bool linear_head_supported(const ConvArgs& a, hc_dtype dt);
 hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
 hc_status launch_conv_tc(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
@@ -320,6 +322,14 @@ __device__ __forceinline__ void cp_async_8(uint32_t dst, const void* src, bool v
 // count includes it).
 __device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+// Wait until at most N of this thread's committed groups are in flight.
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
