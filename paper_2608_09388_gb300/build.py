@@ -2,8 +2,10 @@
 
 Each .cu under csrc/ is compiled to an object in parallel with nvcc
 (-gencode arch=compute_103a,code=sm_103a) and the objects are linked into
-``_build/libhc.so`` with the CUDA runtime linked statically. A build is
-skipped when the library is newer than every source and header.
+``_build/libhc.so`` with the CUDA runtime linked statically. The Python
+binding's extension module (csrc/binding.cpp) is compiled beside them against
+torch's headers and linked to libhc. A build is skipped when both are newer than
+every source and header.
 """
 from __future__ import annotations
 
@@ -12,6 +14,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -19,6 +22,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libhc.so")
+NATIVE = os.path.join(BUILD, "_hc_native.so")
+BINDING = os.path.join(CSRC, "binding.cpp")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -34,15 +39,33 @@ def sources():
 
 
 def _inputs():
-    return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
+    return sources() + [BINDING] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
         os.path.join(INCLUDE, "*.h")) + [os.path.abspath(__file__)]
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     return all(os.path.getmtime(p) <= t for p in _inputs())
+
+
+def _native_commands(nvcc: str, obj: str, out: str):
+    """The binding's compile and link commands (host compiler)."""
+    import torch
+
+    tdir = os.path.dirname(os.path.abspath(torch.__file__))
+    tlib = os.path.join(tdir, "lib")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    comp = ["g++", "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={abi}", "-I", INCLUDE,
+            "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(tdir, "include"),
+            "-isystem", os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+            "-isystem", cuda, "-c", BINDING, "-o", obj]
+    link = ["g++", "-shared", "-o", out, obj, "-L", tlib, "-ltorch_python", "-ltorch_cpu",
+            "-lc10_cuda", "-lc10", "-L", BUILD, "-lhc", "-Wl,-rpath,$ORIGIN",
+            f"-Wl,-rpath,{tlib}"]
+    return comp, link
 
 
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
@@ -61,13 +84,24 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
         r = subprocess.run([nvcc, *flags, "-c", src, "-o", obj], capture_output=True, text=True)
         return src, obj, r
 
+    native_obj = os.path.join(objdir, "binding.cpp.o")
+    native_tmp = NATIVE + f".{os.getpid()}.tmp"
+    native_comp, native_link = _native_commands(nvcc, native_obj, native_tmp)
+
+    def run(cmd, what):
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"{what} failed:\n{r.stdout}\n{r.stderr}")
+
     objs, logs = [], []
-    with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 4)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(12, os.cpu_count() or 4)) as ex:
+        native = ex.submit(run, native_comp, "compiling the binding")
         for src, obj, r in ex.map(one, sources()):
             logs.append(f"== {os.path.basename(src)}\n{r.stdout}{r.stderr}")
             if r.returncode != 0:
                 raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")
             objs.append(obj)
+        native.result()
     with open(os.path.join(BUILD, "nvcc.log"), "w") as f:
         f.write("\n".join(logs))
     tmp = LIB + f".{os.getpid()}.tmp"
@@ -75,6 +109,8 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    run(native_link, "linking the binding")
+    os.replace(native_tmp, NATIVE)
     return LIB
 
 

@@ -5,15 +5,24 @@ tensors (device memory) plus an optional stream (default: torch's current
 stream). Every step of the computation runs in libhc's CUDA kernels; there is
 no host or CPU fallback. If the library has not been built, or no GPU is
 present, the calls raise instead of computing anything.
+
+The tensors are read and checked by a small extension module
+(csrc/binding.cpp, built beside libhc): through ctypes a call cost 11 us of
+host time, more than most small layers take on the GPU; it costs 2.3 us here
+(the launch included).
+load_library() still hands out libhc itself through ctypes, for callers with
+raw pointers.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import threading
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(PKG, "_build", "libhc.so")
+NATIVE_PATH = os.path.join(PKG, "_build", "_hc_native.so")
 
 HC_OK, HC_ERR_INVALID_ARG, HC_ERR_UNSUPPORTED, HC_ERR_CAPACITY = 0, 1, 2, 3
 HC_ERR_INVALID_INDEX, HC_ERR_TIMEOUT, HC_ERR_CUDA = 4, 5, 6
@@ -95,24 +104,23 @@ def load_library(path: str | None = None):
         return lib
 
 
-def _p(t):
-    if t is None:
-        return None
-    if not t.is_cuda:
-        raise ValueError("libhc takes device tensors")
-    if not t.is_contiguous():
-        raise ValueError("libhc takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+_native = None  # the extension module, once loaded
 
 
-def _p_host_ok(t):
-    """A device tensor, or a pinned host tensor (read by the kernel over the
-    host link under unified addressing)."""
-    if t is not None and not t.is_cuda and t.is_pinned():
-        if not t.is_contiguous():
-            raise ValueError("libhc takes contiguous tensors")
-        return ctypes.c_void_p(t.data_ptr())
-    return _p(t)
+def _load_native():
+    global _native
+    load_library()
+    with _lock:
+        if _native is None:
+            import torch  # noqa: F401  (the extension uses its libraries)
+            if not os.path.exists(NATIVE_PATH):
+                raise RuntimeError(f"libhc's binding is not built ({NATIVE_PATH} missing): run "
+                                   "__graft_entry__.build()")
+            spec = importlib.util.spec_from_file_location("_hc_native", NATIVE_PATH)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+            _native = module
+        return _native
 
 
 def _s(stream):
@@ -120,15 +128,6 @@ def _s(stream):
     if stream is None:
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
-
-
-def _dt(t):
-    import torch
-    if t.dtype == torch.float32:
-        return HC_F32
-    if t.dtype == torch.bfloat16:
-        return HC_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
 
 
 def _check(status: int, where: str):
@@ -140,50 +139,47 @@ def _check(status: int, where: str):
 def hc_mask_compact(mask, coords, row_of, batch_offsets, count, stream=None):
     """mask uint8 [B, V] -> coords int32 [B*V, 2], row_of int32 [B, V] (or None),
     batch_offsets int32 [B+1] (or None), count int32 [1]."""
-    B, V = mask.shape
-    _check(load_library().hc_mask_compact(_p(mask), B, V, _p(coords), _p(row_of),
-                                          _p(batch_offsets), _p(count), _s(stream)),
-           "hc_mask_compact")
+    status = (_native or _load_native()).hc_mask_compact(
+        mask, coords, row_of, batch_offsets, count, stream)
+    if status:
+        _check(status, "hc_mask_compact")
 
 
 def hc_mask_compact_static(mask, coords, row_of, batch_offsets, count, stream=None):
     """hc_mask_compact without any device allocation (fixed in-library
     scratch; masks up to HC_STATIC_MAX_MASK_BYTES bytes)."""
-    B, V = mask.shape
-    _check(load_library().hc_mask_compact_static(_p(mask), B, V, _p(coords), _p(row_of),
-                                                 _p(batch_offsets), _p(count), _s(stream)),
-           "hc_mask_compact_static")
+    status = (_native or _load_native()).hc_mask_compact_static(
+        mask, coords, row_of, batch_offsets, count, stream)
+    if status:
+        _check(status, "hc_mask_compact_static")
 
 
 def hc_sparse_spiral_conv_fwd(x, x_layout, coords, row_of, count, spiral, B, V, W, bias, act, y,
                               stream=None):
     """Sparse spiral conv; x dense [B, V, C_in] or compact [., C_in]; W [L*C_in, C_out];
     y [B*V, C_out] capacity (rows 0..N'-1 written)."""
-    L = spiral.shape[1]
-    C_in = x.shape[-1]
-    C_out = W.shape[1]
-    _check(load_library().hc_sparse_spiral_conv_fwd(
-        _p(x), x_layout, _dt(x), _p(coords), _p(row_of), _p(count), _p(spiral), B, V, L, C_in,
-        C_out, _p(W), _p(bias), act, _p(y), _s(stream)), "hc_sparse_spiral_conv_fwd")
+    status = (_native or _load_native()).hc_sparse_spiral_conv_fwd(
+        x, x_layout, coords, row_of, count, spiral, B, V, W, bias, act, y, stream)
+    if status:
+        _check(status, "hc_sparse_spiral_conv_fwd")
 
 
 def hc_conv_rulebook(coords, row_of, count, spiral, B, V, x_layout, rulebook, stream=None):
     """Eq. 4 mapping: rulebook int32 [L, B*V] of input rows per (slot, active row)."""
-    L = spiral.shape[1]
-    _check(load_library().hc_conv_rulebook(_p(coords), _p(row_of), _p(count), _p(spiral), B, V, L,
-                                           x_layout, _p(rulebook), _s(stream)),
-           "hc_conv_rulebook")
+    status = (_native or _load_native()).hc_conv_rulebook(
+        coords, row_of, count, spiral, B, V, x_layout, rulebook, stream)
+    if status:
+        _check(status, "hc_conv_rulebook")
 
 
 def hc_mask_compact_rulebook(mask, spiral, x_layout, coords, row_of, batch_offsets, count,
                              rulebook, stream=None):
     """hc_mask_compact then hc_conv_rulebook in one call (fused kernels where
     the frame fits): mask uint8 [B, V], spiral int32 [V, L]."""
-    B, V = mask.shape
-    L = spiral.shape[1]
-    _check(load_library().hc_mask_compact_rulebook(
-        _p(mask), B, V, _p(spiral), L, x_layout, _p(coords), _p(row_of), _p(batch_offsets),
-        _p(count), _p(rulebook), _s(stream)), "hc_mask_compact_rulebook")
+    status = (_native or _load_native()).hc_mask_compact_rulebook(
+        mask, spiral, x_layout, coords, row_of, batch_offsets, count, rulebook, stream)
+    if status:
+        _check(status, "hc_mask_compact_rulebook")
 
 
 def hc_sparse_conv_rulebook_fwd(x, rulebook, count, W, bias, act, y, coords=None, out=None,
@@ -191,49 +187,36 @@ def hc_sparse_conv_rulebook_fwd(x, rulebook, count, W, bias, act, y, coords=None
     """Sparse conv through a rulebook [L, capacity]: x [x_rows, C_in] (or [B, V, C_in]),
     W [L*C_in, C_out], y [capacity, C_out] or None; out [B, V, C_out] (fused scatter at
     coords) or None."""
-    L, capacity = rulebook.shape
-    C_in = x.shape[-1]
-    x_rows = x.numel() // C_in
-    C_out = W.shape[1]
-    B, V = (out.shape[0], out.shape[1]) if out is not None else (0, 0)
-    _check(load_library().hc_sparse_conv_rulebook_fwd(
-        _p(x), _dt(x if y is None else y), x_rows, _p(rulebook), _p(count), capacity, L, C_in,
-        C_out, _p(W), _p(bias), act, _p(y), _p(coords), B, V, _p(out), _s(stream)),
-        "hc_sparse_conv_rulebook_fwd")
+    status = (_native or _load_native()).hc_sparse_conv_rulebook_fwd(
+        x, rulebook, count, W, bias, act, y, None, coords, out, stream)
+    if status:
+        _check(status, "hc_sparse_conv_rulebook_fwd")
 
 
 def hc_sparse_conv_rulebook_fwd_hint(x, rulebook, count, W, bias, act, y, rows_hint,
                                      coords=None, out=None, stream=None):
     """hc_sparse_conv_rulebook_fwd with a host-side estimate of N' (an int >= 0,
     0 = unknown) that only chooses the tensor-core tiling; same results."""
-    L, capacity = rulebook.shape
-    C_in = x.shape[-1]
-    x_rows = x.numel() // C_in
-    C_out = W.shape[1]
-    B, V = (out.shape[0], out.shape[1]) if out is not None else (0, 0)
-    _check(load_library().hc_sparse_conv_rulebook_fwd_hint(
-        _p(x), _dt(x if y is None else y), x_rows, _p(rulebook), _p(count), capacity, L, C_in,
-        C_out, _p(W), _p(bias), act, _p(y), _p(coords), B, V, _p(out), int(rows_hint),
-        _s(stream)), "hc_sparse_conv_rulebook_fwd_hint")
+    status = (_native or _load_native()).hc_sparse_conv_rulebook_fwd(
+        x, rulebook, count, W, bias, act, y, int(rows_hint), coords, out, stream)
+    if status:
+        _check(status, "hc_sparse_conv_rulebook_fwd_hint")
 
 
 def hc_sparse_linear_fwd(x, count, W, bias, act, y, stream=None):
     """Linear layer on compact rows: x [capacity, C_in], W [C_in, C_out], y [capacity, C_out]."""
-    capacity, C_in = x.shape
-    C_out = W.shape[1]
-    _check(load_library().hc_sparse_linear_fwd(
-        _p(x), _dt(x), _p(count), capacity, C_in, C_out, _p(W), _p(bias), act, _p(y),
-        _s(stream)), "hc_sparse_linear_fwd")
+    status = (_native or _load_native()).hc_sparse_linear_fwd(x, count, W, bias, act, y, stream)
+    if status:
+        _check(status, "hc_sparse_linear_fwd")
 
 
 def hc_sparse_group_norm_fwd(x, batch_offsets, G, eps, gamma, beta, act, y, stream=None):
     """Group norm of compact rows x [capacity, C], per frame (batch_offsets
     [B+1]) and group of C/G channels; y may be x."""
-    capacity, C = x.shape
-    B = batch_offsets.shape[0] - 1
-    _check(load_library().hc_sparse_group_norm_fwd(
-        _p(x), _dt(x), _p(batch_offsets), B, capacity, C, G, float(eps), _p(gamma), _p(beta),
-        act, _p(y), _s(stream)), "hc_sparse_group_norm_fwd")
+    status = (_native or _load_native()).hc_sparse_group_norm_fwd(
+        x, batch_offsets, G, eps, gamma, beta, act, y, stream)
+    if status:
+        _check(status, "hc_sparse_group_norm_fwd")
 
 
 def hc_sparse_conv_gn_fwd(x, rulebook, count, W, bias, coords, batch_offsets, G, eps, gamma,
@@ -241,23 +224,18 @@ def hc_sparse_conv_gn_fwd(x, rulebook, count, W, bias, coords, batch_offsets, G,
     """Sparse conv through a rulebook [L, capacity], then group norm per frame
     (batch_offsets [B+1]) and group of C_out/G channels, then act: y
     [capacity, C_out]."""
-    L, capacity = rulebook.shape
-    C_in = x.shape[-1]
-    x_rows = x.numel() // C_in
-    C_out = W.shape[1]
-    B = batch_offsets.shape[0] - 1
-    _check(load_library().hc_sparse_conv_gn_fwd(
-        _p(x), _dt(y), x_rows, _p(rulebook), _p(count), capacity, L, C_in, C_out, _p(W),
-        _p(bias), _p(coords), _p(batch_offsets), B, G, float(eps), _p(gamma), _p(beta), act,
-        _p(y), _s(stream)), "hc_sparse_conv_gn_fwd")
+    status = (_native or _load_native()).hc_sparse_conv_gn_fwd(
+        x, rulebook, count, W, bias, coords, batch_offsets, G, eps, gamma, beta, act, y, stream)
+    if status:
+        _check(status, "hc_sparse_conv_gn_fwd")
 
 
 def hc_conv_rulebook_transpose(rulebook, count, x_rows, row_ptr, taps, stream=None):
     """Taps reading each input row (keys n*L + l, ascending) from a rulebook [L, capacity]."""
-    L, capacity = rulebook.shape
-    _check(load_library().hc_conv_rulebook_transpose(_p(rulebook), _p(count), capacity, L, x_rows,
-                                                     _p(row_ptr), _p(taps), _s(stream)),
-           "hc_conv_rulebook_transpose")
+    status = (_native or _load_native()).hc_conv_rulebook_transpose(
+        rulebook, count, x_rows, row_ptr, taps, stream)
+    if status:
+        _check(status, "hc_conv_rulebook_transpose")
 
 
 def hc_sparse_conv_rulebook_bwd(x, rulebook, count, W, y, dy, act, row_ptr=None, taps=None,
@@ -265,64 +243,57 @@ def hc_sparse_conv_rulebook_bwd(x, rulebook, count, W, y, dy, act, row_ptr=None,
     """Gradients of the rulebook conv. x [x_rows, C_in] (or [B, V, C_in]);
     y, dy [capacity, C_out]; dx like x (or None); dW [L*C_in, C_out] and
     dbias [C_out] fp32 (or None)."""
-    L, capacity = rulebook.shape
-    C_in = x.shape[-1]
-    x_rows = x.numel() // C_in
-    C_out = W.shape[1]
-    _check(load_library().hc_sparse_conv_rulebook_bwd(
-        _p(x), _dt(x), x_rows, _p(rulebook), _p(count), capacity, L, C_in, C_out, _p(W), _p(y),
-        _p(dy), act, _p(row_ptr), _p(taps), _p(dx), _p(dW), _p(dbias), _s(stream)),
-        "hc_sparse_conv_rulebook_bwd")
+    status = (_native or _load_native()).hc_sparse_conv_rulebook_bwd(
+        x, rulebook, count, W, y, dy, act, row_ptr, taps, dx, dW, dbias, stream)
+    if status:
+        _check(status, "hc_sparse_conv_rulebook_bwd")
 
 
 def hc_mask_score_update(O, alpha_in, alpha_out, sim=None, stream=None):
     """Eq. 3 on mask outputs O [K, N, D]; alpha_in/alpha_out [K] fp32 (may
     be the same tensor); sim [K, K] fp32 or None."""
-    K, N, D = O.shape
-    _check(load_library().hc_mask_score_update(
-        _p(O), _dt(O), K, N, D, _p(alpha_in), _p(alpha_out), _p(sim), _s(stream)),
-        "hc_mask_score_update")
+    status = (_native or _load_native()).hc_mask_score_update(O, alpha_in, alpha_out, sim, stream)
+    if status:
+        _check(status, "hc_mask_score_update")
 
 
 def hc_mask_select_topk(alpha, kappa, selected, stream=None):
     """Indices of the kappa highest scores into selected [kappa] int32."""
-    _check(load_library().hc_mask_select_topk(_p(alpha), alpha.shape[0], kappa, _p(selected),
-                                              _s(stream)), "hc_mask_select_topk")
+    status = (_native or _load_native()).hc_mask_select_topk(alpha, kappa, selected, stream)
+    if status:
+        _check(status, "hc_mask_select_topk")
 
 
 def hc_kappa_masks(masks, selected, B, out, stream=None):
     """out [B*kappa, V]: frame b*kappa + j = masks[selected[j]] (masks [K, V] uint8)."""
-    K, V = masks.shape
-    _check(load_library().hc_kappa_masks(_p(masks), K, V, _p(selected), selected.shape[0], B,
-                                         _p(out), _s(stream)), "hc_kappa_masks")
+    status = (_native or _load_native()).hc_kappa_masks(masks, selected, B, out, stream)
+    if status:
+        _check(status, "hc_kappa_masks")
 
 
 def hc_gather_rows(x, coords, count, frames_per_sample, y, stream=None):
     """S' of Eq. 2: y[n] = x[f // frames_per_sample, v] for coords[n] = (f, v);
     coords None: y[n] = x row n (x viewed as B_in * V rows), n < count. x or y
     may be a pinned host tensor: only the rows copied cross the host link."""
-    B_in, V, C = x.shape
-    _check(load_library().hc_gather_rows(_p_host_ok(x), _dt(x), B_in, V, C, _p(coords), _p(count),
-                                         y.shape[0], frames_per_sample, _p_host_ok(y), _s(stream)),
-           "hc_gather_rows")
+    status = (_native or _load_native()).hc_gather_rows(
+        x, coords, count, frames_per_sample, y, stream)
+    if status:
+        _check(status, "hc_gather_rows")
 
 
 def hc_scatter_dense(y, coords, row_of, count, B, V, zero_fill, out, stream=None):
     """Compact rows y [., C] -> dense out [B, V, C]."""
-    C = y.shape[-1]
-    _check(load_library().hc_scatter_dense(
-        _p(y), _dt(y), _p(coords), _p(row_of), _p(count), B, V, C, int(zero_fill), _p(out),
-        _s(stream)), "hc_scatter_dense")
+    status = (_native or _load_native()).hc_scatter_dense(
+        y, coords, row_of, count, B, V, int(zero_fill), out, stream)
+    if status:
+        _check(status, "hc_scatter_dense")
 
 
 def hc_spiral_conv_fwd(x, spiral, W, bias, act, y, stream=None):
     """Dense spiral conv over every (b, v): x [B, V, C_in] -> y [B, V, C_out]."""
-    B, V, C_in = x.shape
-    L = spiral.shape[1]
-    C_out = W.shape[1]
-    _check(load_library().hc_spiral_conv_fwd(
-        _p(x), _dt(x), _p(spiral), B, V, L, C_in, C_out, _p(W), _p(bias), act, _p(y),
-        _s(stream)), "hc_spiral_conv_fwd")
+    status = (_native or _load_native()).hc_spiral_conv_fwd(x, spiral, W, bias, act, y, stream)
+    if status:
+        _check(status, "hc_spiral_conv_fwd")
 
 
 def hc_test_set_option(option: int, value: int):
