@@ -30,6 +30,7 @@
 // Frames are located by a kThreads-ary block search of the frame table and
 // read a window of kThreads frames at a time into shared memory; loads are
 // issued a batch ahead of the arithmetic.
+// Many frames take the cluster path further down, which reads x once.
 // The general path (one CTA per (frame, group)) serves every other layout,
 // and small frames (a group slice within its register cache), where one
 // launch beats the two latency-bound row-range launches.
@@ -42,7 +43,7 @@
 // The output may alias the input in both paths. Deterministic, no atomics.
 #include <cuda_bf16.h>
 
-#include <cstdlib>
+#include <mutex>
 
 #include "hc_internal.cuh"
 
@@ -721,6 +722,320 @@ __global__ void __launch_bounds__(kThreads, 4)
     }
 }
 
+// ---- cluster path: one pass over memory ------------------------------------
+// A unit is one frame's rows of one part of the channels (128 bytes of a row,
+// or one whole group where that is wider). The g CTAs of a unit (part of a
+// cluster of kClCtas) split its rows, each keeping its rows in shared memory
+// from the statistics to the normalisation, so that x is read once: a slot of
+// 16 bytes belongs to one thread, which copies it in (cp.async), sums it,
+// normalises it and stores it, and then starts the copy of the next unit's
+// chunk into it. Reads of the next unit thus overlap the writes of this one,
+// and no barrier guards the slots; the block only meets to merge statistics,
+// the CTAs of a unit through each other's shared memory and the cluster's
+// barrier. Rows past kClSlots per thread are read a second time instead. g is
+// the fewest CTAs that hold an average frame, or more where there would be
+// idle ones, chosen on the device from the frame table (the same in every CTA).
+// Two CTAs share an SM, so that one's arithmetic overlaps the other's memory
+// accesses.
+// The issue slots bound it next to memory, hence the packed arithmetic and four
+// chunks to a merge: 64 frames x 10475 x 128 bf16 (343 MB read and written) 112
+// us by the row ranges (two passes over x), 137 us here with a merge per chunk
+// and scalar arithmetic, 96 us as it is (3.6 TB/s; 36 clusters take the 256
+// units in 8 rounds, the last of them nearly empty). At 25% / 5% density 39 /
+// 24 -> 29 / 14 us. 512 threads a CTA: 120 us; three CTAs an SM: 97 us.
+constexpr int kClCtas = 8;
+constexpr int kClThreads = 256;
+constexpr int kClSlots = 24;
+constexpr int kClGroup = 8;  // slots per cp.async group
+constexpr size_t kClSmem = (size_t)kClSlots * kClThreads * 16;
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) {
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// Two fp32 values in one 64-bit register pair: the packed instructions do
+// both in one issue slot, which is what this kernel runs out of first.
+__device__ __forceinline__ uint64_t pk(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpk(uint64_t v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// merge, and onto nothing exactly, whatever nb.
+__device__ __forceinline__ void merge_into(float& n, float& mean, float& m2, float nb, float mb,
+                                           float qb) {
+    if (n == 0.f) n = nb, mean = mb, m2 = qb;
+    else merge(n, mean, m2, nb, mb, qb);
+}
+__device__ __forceinline__ void merge_into_xor(float& n, float& mean, float& m2, int o) {
+    const float nb = __shfl_xor_sync(0xffffffffu, n, o);
+    const float mb = __shfl_xor_sync(0xffffffffu, mean, o);
+    const float qb = __shfl_xor_sync(0xffffffffu, m2, o);
+    merge_into(n, mean, m2, nb, mb, qb);
+}
+
+// Stats of 4 chunks at once: their mean about the first value, then the
+// squares about that mean, one merge (a group of equal values keeps exactly
+// that mean and M2 = 0, as with add_chunk).
+template <int VEC, class Raw, class CK>
+__device__ __forceinline__ void add_four(Stats& st, const Raw (&raw)[4]) {
+    constexpr int N = 4 * VEC;
+    uint64_t v[N / 2];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float f[VEC];
+        CK::unpack(raw[c], f);
+#pragma unroll
+        for (int k = 0; k < VEC / 2; ++k) v[c * (VEC / 2) + k] = pk(f[2 * k], f[2 * k + 1]);
+    }
+    float first, other;
+    unpk(v[0], first, other);
+    const uint64_t shift = pk(-first, -first);
+    uint64_t s0 = add2(v[0], shift), s1 = add2(v[1], shift);
+#pragma unroll
+    for (int k = 2; k < N / 2; k += 2) {
+        s0 = add2(s0, add2(v[k], shift));
+        s1 = add2(s1, add2(v[k + 1], shift));
+    }
+    float a, b;
+    unpk(add2(s0, s1), a, b);
+    const float cm = first + (a + b) * (1.f / N);
+    const uint64_t off = pk(-cm, -cm);
+    uint64_t q0 = 0, q1 = 0;  // +0, +0
+#pragma unroll
+    for (int k = 0; k < N / 2; k += 2) {
+        const uint64_t d0 = add2(v[k], off), d1 = add2(v[k + 1], off);
+        q0 = fma2(d0, d0, q0);
+        q1 = fma2(d1, d1, q1);
+    }
+    unpk(add2(q0, q1), a, b);
+    const float nn = st.n + (float)N;
+    const float d = cm - st.mean;
+    const float r = (float)N * __frcp_rn(nn);
+    st.mean = fmaf(d, r, st.mean);
+    st.m2 += (a + b) + d * d * st.n * r;
+    st.n = nn;
+}
+
+template <typename T, int ACT>
+__global__ void __launch_bounds__(kClThreads, 2)
+    gn_cluster_kernel(const T* x, const int32_t* __restrict__ offsets, int B, int C, int pc_max, int cpc,
+                      long long capacity, float eps, const float* __restrict__ gamma,
+                      const float* __restrict__ beta, T* y, unsigned* status) {
+    constexpr int VEC = 16 / (int)sizeof(T);
+    using CK = Chunk<T, VEC>;
+    using Raw = typename CK::Raw;
+    constexpr int kWarps = kClThreads / 32;
+    extern __shared__ __align__(16) uint8_t slots[];
+    __shared__ float s_red[kWarps][32][3];
+    __shared__ float s_part[2][32][3];  // this CTA's sums of the unit, by round parity
+    __shared__ float s_mu[32], s_inv[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int rank = blockIdx.x % kClCtas, cluster = blockIdx.x / kClCtas;
+    const int clusters = gridDim.x / kClCtas;
+    pdl_wait();
+    pdl_trigger();
+    const long long o0 = __ldg(offsets), oB = __ldg(offsets + B);
+    // frames must be in order (each CTA checks a share of the table)
+    for (long long i = (long long)blockIdx.x * kClThreads + t; i < B;
+         i += (long long)gridDim.x * kClThreads)
+        if (__ldg(offsets + i + 1) < __ldg(offsets + i)) report(status, kErrIndex);
+    if (o0 < 0 || oB < o0 || oB > capacity) {
+        if (t == 0 && blockIdx.x == 0) report(status, kErrIndex);
+        return;  // every CTA alike
+    }
+    // half-width parts where the slots of a cluster do not hold an average
+    // frame at full width
+    const long long avg = (oB - o0 + B - 1) / B;
+    int pc = pc_max;
+    if (avg > (long long)kClCtas * kClSlots * (kClThreads / pc) && pc / 2 >= cpc && pc / 2 >= 4) pc /= 2;
+    const int parts = C / VEC / pc;
+    const int rpp = kClThreads / pc;  // rows of a slot
+    const long long units = (long long)B * parts;
+    int g = 1;
+    while (g < kClCtas && (avg > (long long)g * kClSlots * rpp || units * g * 2 <= gridDim.x)) g *= 2;
+    const int per = kClCtas / g;  // units of a cluster at a time
+    const int sub = rank / g, r = rank - sub * g;
+    const long long rounds = (units + (long long)clusters * per - 1) / ((long long)clusters * per);
+    const int tc = t % pc, tr = t / pc;
+    const int groups = pc / cpc;
+    const uint32_t slot0 = smem_u32(slots) + (uint32_t)t * 16u;
+
+    // a round's unit: this thread's first chunk, and how many rows of the CTA's
+    // share lie at and after it (slot i holds the chunk i * rpp rows further)
+    struct Share {
+        long long at;  // element offset of the first chunk
+        int rows, col;
+    };
+    auto locate = [&](long long round) {
+        Share sh{0, 0, tc * VEC};
+        const long long u = (round * clusters + cluster) * per + sub;
+        if (round >= rounds || u >= units) return sh;
+        const int b = (int)(u / parts);
+        sh.col = ((int)(u - (long long)b * parts) * pc + tc) * VEC;
+        const long long f0 = __ldg(offsets + b), f1 = __ldg(offsets + b + 1);
+        if (f0 < o0 || f1 < f0 || f1 > oB) return sh;  // reported above, or outside the span
+        const long long n = f1 - f0, s0 = f0 + n * r / g, s1 = f0 + n * (r + 1) / g;
+        sh.rows = (int)(s1 - s0) - tr;
+        sh.at = (s0 + tr) * C + sh.col;
+        return sh;
+    };
+    const long long step = (long long)rpp * C;
+    auto copies = [&](const Share& sh, int i0, int i1) {
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i)
+            if (i * rpp < sh.rows)
+                cp_async_16(slot0 + (uint32_t)i * (kClThreads * 16u), x + sh.at + i * step, true);
+        cp_async_commit();
+    };
+    auto slot = [&](int i) {
+        return *reinterpret_cast<const Raw*>(slots + (size_t)(i * kClThreads + t) * 16);
+    };
+
+    Share cur = locate(0);
+    for (int i = 0; i < kClSlots; i += kClGroup) copies(cur, i, i + kClGroup);
+    for (long long round = 0; round < rounds; ++round) {
+        const int par = (int)(round & 1);
+        // statistics
+        Stats st;
+        const int mine = cur.rows > 0 ? (cur.rows + rpp - 1) / rpp : 0;  // chunks of this thread
+        auto add = [&](int i0) {
+            int i = i0;
+            for (; i + 4 <= i0 + kClGroup && i + 4 <= mine; i += 4) {
+                const Raw raw[4] = {slot(i), slot(i + 1), slot(i + 2), slot(i + 3)};
+                add_four<VEC, Raw, CK>(st, raw);
+            }
+            for (; i < i0 + kClGroup && i < mine; ++i) {
+                float v[VEC];
+                CK::unpack(slot(i), v);
+                st.template add_chunk<VEC>(v);
+            }
+        };
+        static_assert(kClSlots == 3 * kClGroup, "three copy groups a unit");
+        cp_async_wait_group<2>();
+        add(0);
+        cp_async_wait_group<1>();
+        add(kClGroup);
+        cp_async_wait_group<0>();
+        add(2 * kClGroup);
+        // chunks without a slot
+        int ex = kClSlots;
+        for (; ex + 4 <= mine; ex += 4) {
+            Raw raw[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) raw[k] = CK::load(x + cur.at + (ex + k) * step);
+            add_four<VEC, Raw, CK>(st, raw);
+        }
+        for (; ex < mine; ++ex) {
+            float v[VEC];
+            CK::unpack(CK::load(x + cur.at + ex * step), v);
+            st.template add_chunk<VEC>(v);
+        }
+        // lanes of a group (cpc chunk columns, every row of the warp)
+        for (int o = 1; o < cpc; o <<= 1) merge_into_xor(st.n, st.mean, st.m2, o);
+        for (int o = pc; o < 32; o <<= 1) merge_into_xor(st.n, st.mean, st.m2, o);
+        if (lane < pc && lane % cpc == 0) {
+            float* e = s_red[warp][lane / cpc];
+            e[0] = st.n, e[1] = st.mean, e[2] = st.m2;
+        }
+        __syncthreads();
+        if (t < groups) {
+            float n = 0.f, mean = 0.f, m2 = 0.f;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w)
+                merge_into(n, mean, m2, s_red[w][t][0], s_red[w][t][1], s_red[w][t][2]);
+            s_part[par][t][0] = n, s_part[par][t][1] = mean, s_part[par][t][2] = m2;
+        }
+        if (g > 1) cluster_sync();
+        else __syncthreads();
+        for (int q = warp; q < groups; q += kWarps) {
+            float n = 0.f, mean = 0.f, m2 = 0.f;
+            if (lane < g) {
+                const uint32_t e = smem_u32(&s_part[par][q][0]);
+                n = ld_cluster(e, sub * g + lane);
+                mean = ld_cluster(e + 4u, sub * g + lane);
+                m2 = ld_cluster(e + 8u, sub * g + lane);
+            }
+            for (int o = 1; o < g; o <<= 1) merge_into_xor(n, mean, m2, o);
+            if (lane == 0) {
+                s_mu[q] = mean;
+                s_inv[q] = 1.f / sqrtf(m2 / n + eps);
+            }
+        }
+        __syncthreads();
+        const float mu = s_mu[tc / cpc], inv = s_inv[tc / cpc];
+        const uint64_t off = pk(-mu, -mu);
+        uint64_t sc[VEC / 2], be[VEC / 2];
+#pragma unroll
+        for (int k = 0; k < VEC / 2; ++k) {
+            const int c = cur.col + 2 * k;
+            sc[k] = gamma ? pk(inv * __ldg(gamma + c), inv * __ldg(gamma + c + 1)) : pk(inv, inv);
+            be[k] = beta ? pk(__ldg(beta + c), __ldg(beta + c + 1)) : 0;
+        }
+        auto finish = [&](Raw raw, int i) {
+            float v[VEC];
+            CK::unpack(raw, v);
+#pragma unroll
+            for (int k = 0; k < VEC / 2; ++k) {
+                const uint64_t z = fma2(add2(pk(v[2 * k], v[2 * k + 1]), off), sc[k], be[k]);
+                float z0, z1;
+                unpk(z, z0, z1);
+                if (ACT == HC_ACT_ELU) {  // max(z, 0) + (exp(min(z, 0)) - 1)
+                    const uint64_t e = pk(__expf(fminf(z0, 0.f)), __expf(fminf(z1, 0.f)));
+                    unpk(add2(pk(fmaxf(z0, 0.f), fmaxf(z1, 0.f)), add2(e, pk(-1.f, -1.f))), v[2 * k],
+                         v[2 * k + 1]);
+                } else {
+                    v[2 * k] = act_fixed<ACT>(z0);
+                    v[2 * k + 1] = act_fixed<ACT>(z1);
+                }
+            }
+            Raw packed;
+            CK::store(reinterpret_cast<T*>(&packed), v);
+            __stcs(reinterpret_cast<uint4*>(y + cur.at + i * step), as_u4(packed));
+        };
+        ex = kClSlots;
+        for (; ex + 4 <= mine; ex += 4) {
+            Raw raw[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) raw[k] = CK::load(x + cur.at + (ex + k) * step);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) finish(raw[k], ex + k);
+        }
+        for (; ex < mine; ++ex) finish(CK::load(x + cur.at + ex * step), ex);
+        // every slot: this unit's chunk out, then the next unit's on its way in
+        const Share next = locate(round + 1);
+        for (int i0 = 0; i0 < kClSlots; i0 += kClGroup) {
+#pragma unroll 4
+            for (int i = i0; i < i0 + kClGroup; ++i)
+                if (i < mine) finish(slot(i), i);
+            copies(next, i0, i0 + kClGroup);
+        }
+        cur = next;
+    }
+    if (g > 1) cluster_sync();  // no CTA leaves while another reads its sums
+}
+
 long long fast_grid(const DeviceCtx* ctx, long long capacity) {
     // ranges of at least ~64 rows; 2 CTAs per SM at most (the kernels' bound)
     long long grid = (capacity + 63) / 64;
@@ -747,6 +1062,70 @@ hc_status launch_fast(const DeviceCtx* ctx, const void* x, const int32_t* offset
 }
 
 
+// The part of a row that a unit of the cluster path covers, in 16-byte chunks
+// (0: the path does not take this layout): 128 bytes, or one group where that
+// is wider, and both whole powers of two of chunks, one thread of a warp each.
+int cluster_part_chunks(int C, int cpg, int vec) {
+    if (cpg % vec != 0) return 0;
+    const int cpc = cpg / vec, cpr = C / vec;
+    if ((cpc & (cpc - 1)) != 0 || cpc > 32) return 0;
+    const int pc = cpc > 8 ? cpc : 8;
+    return cpr % pc == 0 ? pc : 0;
+}
+
+template <typename T, int ACT>
+hc_status launch_cluster(const DeviceCtx* ctx, const T* x, const int32_t* offsets, int B,
+                         long long capacity, int C, int pc, int cpc, float eps, const float* gamma,
+                         const float* beta, T* y, cudaStream_t s, bool& taken) {
+    auto kernel = gn_cluster_kernel<T, ACT>;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClCtas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = kClSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    // clusters that fit the device at a time (0: none), looked up once
+    static std::mutex mutex;
+    static int resident[64] = {};
+    static bool known[64] = {};
+    int clusters = 0;
+    {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!known[ctx->device]) {
+            hc_status st = check_cuda(
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem),
+                "cudaFuncSetAttribute(gn_cluster_kernel)");
+            if (st == HC_OK)
+                st = check_cuda(
+                    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1),
+                    "cudaFuncSetAttribute(gn_cluster_kernel)");
+            if (st != HC_OK) return st;
+            cfg.gridDim = dim3(kClCtas);
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            resident[ctx->device] = n;
+            known[ctx->device] = true;
+        }
+        clusters = resident[ctx->device];
+    }
+    taken = clusters > 0;
+    if (!taken) return HC_OK;
+    cfg.gridDim = dim3((unsigned)(clusters * kClCtas));
+    cfg.numAttrs = 2;
+    return check_cuda(cudaLaunchKernelEx(&cfg, kernel, x, offsets, B, C, pc, cpc, capacity, eps,
+                                         gamma, beta, y, ctx->status),
+                      "gn_cluster_kernel");
+}
+
 template <typename T>
 hc_status launch_typed(const DeviceCtx* ctx, const void* x, const int32_t* offsets, int B,
                        long long capacity, int C, int G, float eps, const float* gamma,
@@ -772,6 +1151,28 @@ hc_status launch_typed(const DeviceCtx* ctx, const void* x, const int32_t* offse
     const bool force_rows = forced == 2;
     const bool fast_rows = aligned && cpr >= 1 && cpr <= kThreads && (cpr & (cpr - 1)) == 0 &&
                            G <= kMaxGroupsFast && !force_slice && (force_rows || !small_frames);
+    // The cluster path reads x once. It needs enough units (frames x parts) to
+    // give every cluster work, else the row ranges spread few large frames over
+    // the whole GPU (two 10475-row frames: the same 22.6 us either way). Small
+    // frames stay with one CTA per (frame, group) while those are one wave, 4
+    // an SM (64 frames x 8 groups: 6-8 us there, 10 us here); past it the
+    // cluster path is ahead (256 frames x 8 groups, 655 rows: 26.8 us there,
+    // 20.5 us here; 128 x 8: 16.8 and 13.6; 100 x 8: 14.4 either way).
+    const int pc = aligned ? cluster_part_chunks(C, cpg, kVec) : 0;
+    const bool one_wave = small_frames && (long long)B * G <= 4ll * ctx->num_sms;
+    if (pc > 0 && forced == 0 && !one_wave && (long long)B * (cpr / pc) >= 16) {
+        bool taken = false;
+        const int cpc = cpg / kVec;
+        const hc_status st =
+            act == HC_ACT_ELU ? launch_cluster<T, HC_ACT_ELU>(ctx, (const T*)x, offsets, B, capacity, C, pc, cpc,
+                                                              eps, gamma, beta, (T*)y, s, taken)
+            : act == HC_ACT_RELU
+                ? launch_cluster<T, HC_ACT_RELU>(ctx, (const T*)x, offsets, B, capacity, C, pc, cpc, eps,
+                                                 gamma, beta, (T*)y, s, taken)
+                : launch_cluster<T, HC_ACT_NONE>(ctx, (const T*)x, offsets, B, capacity, C, pc, cpc, eps,
+                                                 gamma, beta, (T*)y, s, taken);
+        if (st != HC_OK || taken) return st;
+    }
     if (fast_rows && cpg % kVec == 0)
         return launch_fast<T, kVec, 1>(ctx, x, offsets, B, capacity, C, G, eps, gamma, beta, act,
                                        y, s);
