@@ -10,12 +10,11 @@
 // fixed order, no floating-point atomics):
 //   act_bwd_kernel      dz (stored in the layer dtype) and per-block column
 //                       sums of dz in fp32 (act_bwd_vec_kernel: 16-byte
-//                       chunks); further blocks of the same launch count the
-//                       present taps per (slot, row unit) for wgrad and the
-//                       taps of the transposed mapping per slot for dgrad.
+//                       chunks); further blocks of the same launch list
+//                       the present taps per (slot, row unit) for wgrad and
+//                       count the taps of the transposed mapping per slot for dgrad.
 //   wgrad               dW_l = sum over the slot's present taps: equal runs
-//                       of taps per CTA, compacted from the rulebook on the
-//                       fly, x and dz rows gathered; tcgen05 (fp32
+//                       of the lists per CTA, x and dz rows gathered; tcgen05 (fp32
 //                       accumulators in TMEM) or CUDA cores (fp32).
 //                       bwd_collect adds a slot's runs and dbias's blocks.
 //   dgrad               tap_slots: the taps of the transposed mapping listed
@@ -24,9 +23,8 @@
 //                       sums its own, consecutive rows of P, in (n, l) order.
 // The transposed mapping itself: rb_* kernels (counts, exclusive scan, fill,
 // per-row sort).
-#include <cuda_bf16.h>
-
 #include <cuda.h>
+#include <cuda_bf16.h>
 
 #include "hc_internal.cuh"
 
@@ -608,22 +606,23 @@ struct Run {
         const long long end = s_pre[(l + 1) * kUnits];
         return end < p1 ? end : p1;
     }
-    // Entry of the unit lists (see count_taps) of position pos of slot l.
-    __device__ __forceinline__ long long entry(int l, int pos, long long urows,
-                                               long long capacity) const {
-        int lo = l * kUnits, hi = (l + 1) * kUnits - 1;  // last unit with s_pre <= pos
-#pragma unroll
-        for (int step = 0; step < 7; ++step) {
-            const int mid = (lo + hi + 1) >> 1;
-            const bool le = s_pre[mid] <= pos;
-            lo = le ? mid : lo;
-            hi = le ? hi : mid - 1;
+    // Entry of the unit lists (see count_taps) of position pos of slot l. u:
+    // the unit of an earlier position of the slot (or the slot's first), moved
+    // on to pos's: mostly the same one or the next, else searched for.
+    __device__ __forceinline__ long long entry(int l, int pos, long long urows, long long capacity,
+                                               int& u) const {
+        if (s_pre[u + 1] <= pos && s_pre[++u + 1] <= pos) {
+            int lo = u + 1, hi = (l + 1) * kUnits - 1;  // last unit with s_pre <= pos
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_pre[mid] <= pos) lo = mid;
+                else hi = mid - 1;
+            }
+            u = lo;
         }
-        return l * capacity + (lo - l * kUnits) * urows + (pos - s_pre[lo]);
+        return l * capacity + (u - l * kUnits) * urows + (pos - s_pre[u]);
     }
 };
-static_assert(kUnits == 1 << 7, "Run::entry halves a slot's units seven times");
-
 // tcgen05: D[o][c] (M = 128 output channels of dz, N = BC channels of x),
 // both operands MN-major as gathered: per stage kBK taps, dz's rows as up to
 // two and x's as BC / 64 atoms of 64 channels (kBK rows x 128 bytes each,
@@ -636,7 +635,7 @@ static_assert(kUnits == 1 << 7, "Run::entry halves a slot's units seven times");
 // producers' copies.) Warps 0-3 gather
 // with 16-byte cp.async, warp 8 issues the MMAs, warps 4-7 move a finished
 // segment's sums from TMEM to its partial while the next one accumulates.
-// 167k rows, 9 slots, 128 -> 128, 25% present: 146 -> 45 us (two thirds of the
+// 167k rows, 9 slots, 128 -> 128, 25% present: 146 -> 37 us (two thirds of the
 // taps were multiplied as zeros, the lookups' latency was paid per stage);
 // 16.4k rows, 12 slots, 64 -> 128, 84% present: 17.5 -> 18.9 us (the rows of
 // dz are gathered per slot, 24 KB a stage). fp32, 25k rows, 9 slots, 64 -> 128,
@@ -813,13 +812,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs
         int l = 0;
         for (long long pos = run.p0; pos < run.p1 && ok;) {
             const long long end = run.segment(pos, l);
+            int unit[2] = {l * kUnits, l * kUnits};
             for (; pos < end; pos += kBK) {
                 // position pos + i -> entry i; zeros past the segment's end
                 long long src[2];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     const long long p = pos + lane + 32 * i;
-                    src[i] = p < end ? run.entry(l, (int)p, urows, a.capacity) : -1;
+                    src[i] = p < end ? run.entry(l, (int)p, urows, a.capacity, unit[i]) : -1;
                 }
                 if (!mbar_wait(qempty_bar(qt), qph ^ 1u, abort_flag, a.status)) {
                     ok = false;
@@ -956,6 +956,7 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
     int l = 0;
     for (long long pos = run.p0; pos < run.p1;) {
         const long long end = run.segment(pos, l);
+        int unit = l * kUnits;
         float acc[4][8];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -964,7 +965,7 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
         for (; pos < end; pos += kSimtBatch) {
             const int want = end - pos < kSimtBatch ? (int)(end - pos) : kSimtBatch;
             if (t < want) {
-                const int2 e = __ldg(a.unit_list + run.entry(l, (int)pos + t, urows, a.capacity));
+                const int2 e = __ldg(a.unit_list + run.entry(l, (int)pos + t, urows, a.capacity, unit));
                 s_j[t] = e.x - 1;
                 s_n[t] = e.y - 1;
             }
@@ -1507,13 +1508,31 @@ __global__ void __launch_bounds__(kTapThreads, 1)
     }
 }
 
-// CUDA cores: 64 listed taps x 64 channels per item, 4 x 4 per thread over
-// chunks of 32 of C_out (both operands' rows are contiguous along it and
-// are turned round on their way into shared memory).
-constexpr int kTgBM = 64, kTgBN = 64, kTgBK = 32;
+// CUDA cores: 128 listed taps x 64 channels per item, 8 x 4 per thread over
+// chunks of 32 of C_out, the next chunk in registers while one is multiplied.
+// Both operands' rows are contiguous along C_out and are turned round on their
+// way into shared memory: a warp loads 8 values of 4 rows at a time, which are
+// 32-byte pieces in global memory and 32 different banks in shared memory.
+// Shared memory returns one word per lane and clock: 8 x 4 reads 12 for 32
+// multiply-adds (4 x 4 reads 8 for 16: 38 us instead of 35, 25k rows, 64 ->
+// 128, 24% of the taps present).
+constexpr int kTgBM = 128, kTgBN = 64, kTgBK = 32;
 
 template <typename T>
-__global__ void __launch_bounds__(256) tap_gemm_simt_kernel(const TapGemmArgs a) {
+__device__ __forceinline__ void store4(T* dst, const float* v);
+template <>
+__device__ __forceinline__ void store4<float>(float* dst, const float* v) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <>
+__device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* dst, const float* v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+    *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&a),
+                                                *reinterpret_cast<const uint32_t*>(&b));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs a) {
     __shared__ __align__(16) float As[kTgBK][kTgBM + 4];
     __shared__ __align__(16) float Bs[kTgBK][kTgBN + 4];
     __shared__ int s_off[33], s_tile[33], s_e[kTgBM];
@@ -1525,7 +1544,8 @@ __global__ void __launch_bounds__(256) tap_gemm_simt_kernel(const TapGemmArgs a)
     const T* __restrict__ W = static_cast<const T*>(a.W);
     T* __restrict__ P = static_cast<T*>(a.P);
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-    const int kk = t & 31, row = t >> 5;  // loads: k = kk, rows row + 8 i
+    // loads: k = kl + 8 j; taps ra + 4 i, channels rb + 4 i
+    const int kl = t & 7, ra = (t >> 5) * 16 + ((t >> 3) & 3), rb = (t >> 5) * 8 + ((t >> 3) & 3);
     const long long items = (long long)s_tile[a.L] * a.c_tiles;
     int l = 0;
     for (long long w = blockIdx.x; w < items; w += gridDim.x) {
@@ -1534,58 +1554,68 @@ __global__ void __launch_bounds__(256) tap_gemm_simt_kernel(const TapGemmArgs a)
         while (s_tile[l + 1] <= tile) ++l;
         const int first = s_off[l] + (tile - s_tile[l]) * kTgBM, end = s_off[l + 1];
         if (t < kTgBM) s_e[t] = first + t < end ? __ldg(a.list_e + first + t) : -1;
-        int n[8];
+        long long za[4], wb[2];  // first element of this thread's rows, -1: none
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int e = first + row + 8 * i;
-            n[i] = e < end ? __ldg(a.list_n + e) : -1;
+        for (int i = 0; i < 4; ++i) {
+            const int e = first + ra + 4 * i;
+            const int n = e < end ? __ldg(a.list_n + e) : -1;
+            za[i] = n >= 0 ? (long long)n * a.C_out : -1;
         }
-        float acc[4][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 2; ++i) {
+            const int c = c0 + rb + 4 * i;
+            wb[i] = c < a.C_in ? ((long long)l * a.C_in + c) * a.C_out : -1;
+        }
+        float acc[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-        float av[8], bv[8];
+        float av[4][4], bv[2][4];
         auto fetch = [&](int k0) {
-            const int k = k0 + kk;
-            const bool in = k < a.C_out;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                av[i] = in && n[i] >= 0 ? to_f(dz[(long long)n[i] * a.C_out + k]) : 0.f;
-                const int c = c0 + row + 8 * i;
-                bv[i] = in && c < a.C_in ? to_f(W[((long long)l * a.C_in + c) * a.C_out + k]) : 0.f;
+            for (int j = 0; j < 4; ++j) {
+                const int k = k0 + kl + 8 * j;
+                const bool in = k < a.C_out;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) av[i][j] = in && za[i] >= 0 ? to_f(dz[za[i] + k]) : 0.f;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) bv[i][j] = in && wb[i] >= 0 ? to_f(W[wb[i] + k]) : 0.f;
             }
         };
         fetch(0);
         for (int k0 = 0; k0 < a.C_out; k0 += kTgBK) {
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                As[kk][row + 8 * i] = av[i];
-                Bs[kk][row + 8 * i] = bv[i];
+            for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) As[kl + 8 * j][ra + 4 * i] = av[i][j];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) Bs[kl + 8 * j][rb + 4 * i] = bv[i][j];
             }
             __syncthreads();
             if (k0 + kTgBK < a.C_out) fetch(k0 + kTgBK);
-#pragma unroll
+#pragma unroll 8
             for (int k = 0; k < kTgBK; ++k) {
-                const float4 x4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
+                const float4 xa = *reinterpret_cast<const float4*>(&As[k][ty * 8]);
+                const float4 xb = *reinterpret_cast<const float4*>(&As[k][ty * 8 + 4]);
                 const float4 w4 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-                const float xr[4] = {x4.x, x4.y, x4.z, x4.w}, wr[4] = {w4.x, w4.y, w4.z, w4.w};
+                const float xr[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+                const float wr[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < 8; ++i)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xr[i], wr[j], acc[i][j]);
             }
         }
+        // P's rows are whole 16-byte chunks (Cp)
+        const int c = c0 + tx * 4;
+        if (c < a.Cp)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const long long e = s_e[ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int c = c0 + tx * 4 + j;
-                if (e >= 0 && c < a.Cp) P[e * a.Cp + c] = from_f<T>(acc[i][j]);
+            for (int i = 0; i < 8; ++i) {
+                const long long e = s_e[ty * 8 + i];
+                if (e >= 0) store4<T>(P + e * a.Cp + c, acc[i]);
             }
-        }
         __syncthreads();  // s_e is free
     }
 }
@@ -1916,7 +1946,7 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         } else {
             g.c_tiles = (b.C_in + kTgBN - 1) / kTgBN;
             st = launch_pdl(bf ? tap_gemm_simt_kernel<__nv_bfloat16> : tap_gemm_simt_kernel<float>,
-                            dim3((unsigned)(4 * ctx->num_sms)), dim3(256), 0, s,
+                            dim3((unsigned)(2 * ctx->num_sms)), dim3(256), 0, s,
                             "tap_gemm_simt_kernel", g);
         }
         if (st != HC_OK) return st;
