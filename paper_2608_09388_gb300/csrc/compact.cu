@@ -451,24 +451,39 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
     }
     const long long n0 = (long long)off + R0;  // first row of the portion
     unsigned err = 0;
-    for (int i = tid; i < items; i += kMapThreads) {
-        int k;
-        const int l = (int)div32(i, nact, k);
-        const int q = (i - tid) / kMapThreads;
-        int u = -1;
+    // the prefetched entries, then batches of kMapPre in flight (one by one a
+    // portion with more entries paid a round trip for each: the headline layer
+    // 22.5 -> 21.6 us in graph replays; batches of 8: 21.8)
+    for (int i0 = tid; i0 < items; i0 += kMapPre * kMapThreads) {
+        if (i0 != tid) {
 #pragma unroll
-        for (int j = 0; j < kMapPre; ++j)
-            if (q == j) u = u_pre[j];
-        if (q >= kMapPre) u = __ldg(a.spiral + (long long)(v0 + act_v[k]) * L + l);
-        int e = -1;
-        if (u < -1 || u >= V) {
-            err |= kErrIndex;
-        } else if (u >= 0) {
-            bool hit;
-            const int r = rank_of(u, hit);
-            if (hit) e = a.x_layout == HC_LAYOUT_DENSE ? (int)(fb + u) : off + r;
+            for (int q = 0; q < kMapPre; ++q) {
+                const int i = i0 + q * kMapThreads;
+                u_pre[q] = -1;
+                if (i < items) {
+                    int k;
+                    const int l = (int)div32(i, nact, k);
+                    u_pre[q] = __ldg(a.spiral + (long long)(v0 + act_v[k]) * L + l);
+                }
+            }
         }
-        a.rulebook[(long long)l * a.n + n0 + k] = e;
+#pragma unroll
+        for (int q = 0; q < kMapPre; ++q) {
+            const int i = i0 + q * kMapThreads;
+            if (i >= items) break;
+            int k;
+            const int l = (int)div32(i, nact, k);
+            const int u = u_pre[q];
+            int e = -1;
+            if (u < -1 || u >= V) {
+                err |= kErrIndex;
+            } else if (u >= 0) {
+                bool hit;
+                const int r = rank_of(u, hit);
+                if (hit) e = a.x_layout == HC_LAYOUT_DENSE ? (int)(fb + u) : off + r;
+            }
+            a.rulebook[(long long)l * a.n + n0 + k] = e;
+        }
     }
     if (a.row_of)
         for (int p = v0 + tid; p < v1; p += kMapThreads) {
