@@ -829,7 +829,7 @@ def run_group_norm(torch, hc, sets, dev, stream, Wt, bias, G=8):
     nbytes = 2 * x.numel() * 2
     gbs = nbytes / (ms * 1e-3) / 1e9
     out["large"] = {"rows": Bl * Vl, "C": C, "bytes": nbytes, "us": ms * 1e3, "gbs": gbs,
-                    "kernels": "gn_stats_kernel + gn_apply_kernel (contiguous row ranges)",
+                    "kernels": "gn_cluster_kernel (frames kept in shared memory, x read once)",
                     "hbm_frac": gbs / pk["hbm_gbs"],
                     "peak": f"{pk['hbm_gbs']} GB/s ({pk['source']} copy)"}
     st = hc.hc_get_device_status(stream)
@@ -942,8 +942,8 @@ def run_backward(torch, hc, s, w, spiral, Wt, dev, stream):
     return {"workload": WORKLOAD, "active_rows": s.rows, "dtype": "bf16",
             "transpose_us": t_tr, "bwd_us": t_all, "wgrad_part_us": t_w, "dgrad_part_us": t_x,
             "wgrad_tflops": tf, "wgrad_tensor_frac": tf / pk["bf16_tflops"],
-            "kernels": "act_bwd + wgrad_tc_kernel (tcgen05 split-K) + wgrad_reduce; "
-                       "W^T + linear conv (dz W^T) + dgrad gather-sum",
+            "kernels": "act_bwd (+ tap lists) + wgrad_tc_kernel (tcgen05, present taps) + "
+                       "bwd_collect; tap_gemm_tc_kernel + seg_sum_kernel",
             "peak": f"{pk['bf16_tflops']} TFLOP/s ({pk['source']} bf16 burst)"}
 
 

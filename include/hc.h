@@ -176,8 +176,8 @@ hc_status hc_conv_rulebook(const int32_t* coords, const int32_t* row_of, const i
 /*
  * hc_mask_compact_rulebook -- hc_mask_compact followed by hc_conv_rulebook on
  * its output (Eq. 2 and the Eq. 4 indexing matrix), in two kernels when
- * V <= 65535: a count pass, then one pass per (frame, block of 1024
- * vertices) that ranks the frame's mask bytes in shared memory and writes
+ * V <= 65535: a count pass (none for masks of up to 16 KB), then one pass
+ * per (frame, block of 1024 vertices) that ranks the frame's mask bytes in shared memory and writes
  * coords, row_of, batch_offsets, count and the rulebook columns of its
  * active vertices, every tap lookup answered from shared memory. Larger
  * frames run the two operations' own kernels. The results are identical to
@@ -322,7 +322,8 @@ hc_status hc_sparse_conv_gn_fwd(const void* x, hc_dtype dt, int x_rows, const in
  *   taps      [L * capacity] int32
  * Entries outside [-1, x_rows) are skipped and reported
  * (HC_ERR_INVALID_INDEX). Computed once per mask and reused by every layer.
- * Uses the library's per-stream workspace (2 int32 per input row).
+ * Uses the library's per-stream workspace (one int32 per input row and one
+ * per rulebook entry).
  */
 hc_status hc_conv_rulebook_transpose(const int32_t* rulebook, const int32_t* count, int capacity,
                                      int L, int x_rows, int32_t* row_ptr, int32_t* taps,
