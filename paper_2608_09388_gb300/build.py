@@ -4,7 +4,7 @@ Each .cu under csrc/ is compiled to an object in parallel with nvcc
 (-gencode arch=compute_103a,code=sm_103a) and the objects are linked into
 ``_build/libhc.so`` with the CUDA runtime linked statically. The Python
 binding's extension module (csrc/binding.cpp) is compiled beside them against
-torch's headers and linked to libhc. A build is skipped when both are newer than
+torch's headers. A build is skipped when both are newer than
 every source and header.
 """
 from __future__ import annotations
@@ -63,8 +63,7 @@ def _native_commands(nvcc: str, obj: str, out: str):
             "-isystem", os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
             "-isystem", cuda, "-c", BINDING, "-o", obj]
     link = ["g++", "-shared", "-o", out, obj, "-L", tlib, "-ltorch_python", "-ltorch_cpu",
-            "-lc10_cuda", "-lc10", "-L", BUILD, "-lhc", "-Wl,-rpath,$ORIGIN",
-            f"-Wl,-rpath,{tlib}"]
+            "-lc10_cuda", "-lc10", "-ldl", f"-Wl,-rpath,{tlib}"]
     return comp, link
 
 

@@ -4,13 +4,37 @@
 // them; see hc.py for what each function takes. Every function returns the
 // hc_status as an int, or raises ValueError / TypeError where an argument is
 // not one that the binding passes on. No tensor or pointer outlives its call.
+//
+// The module is not linked to libhc: bind() takes the handle of the library
+// that hc.load_library() opened, and every call goes there. The library's
+// error string and device status are its own, so a call into another copy of
+// it would lose them.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <dlfcn.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "hc.h"
 
 namespace {
+
+// clang-format off
+#define HC_CALLS(X) \
+    X(hc_mask_compact) X(hc_mask_compact_static) X(hc_sparse_spiral_conv_fwd) \
+    X(hc_conv_rulebook) X(hc_mask_compact_rulebook) X(hc_sparse_conv_rulebook_fwd) \
+    X(hc_sparse_conv_rulebook_fwd_hint) X(hc_sparse_linear_fwd) X(hc_sparse_group_norm_fwd) \
+    X(hc_sparse_conv_gn_fwd) X(hc_conv_rulebook_transpose) X(hc_sparse_conv_rulebook_bwd) \
+    X(hc_mask_score_update) X(hc_mask_select_topk) X(hc_kappa_masks) X(hc_gather_rows) \
+    X(hc_scatter_dense) X(hc_spiral_conv_fwd)
+// clang-format on
+
+struct Library {
+#define MEMBER(f) decltype(&::f) f;
+    HC_CALLS(MEMBER)
+#undef MEMBER
+};
+Library lib;  // by bind()
+bool bound = false;
 
 struct PyError {};  // a Python exception is set
 
@@ -104,6 +128,10 @@ PyObject* entry(PyObject* const* a, Py_ssize_t n, F&& f) {
         PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
         return nullptr;
     }
+    if (!bound) {
+        PyErr_SetString(PyExc_RuntimeError, "libhc is not bound");
+        return nullptr;
+    }
     try {
         return PyLong_FromLong(f(a));
     } catch (const PyError&) {
@@ -126,7 +154,7 @@ int unlocked(F&& f) {
 using I32 = int32_t;
 #define FN(name) PyObject* name(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 
-template <hc_status (*F)(const uint8_t*, int, int, I32*, I32*, I32*, I32*, hc_stream_t)>
+template <hc_status (*Library::*F)(const uint8_t*, int, int, I32*, I32*, I32*, I32*, hc_stream_t)>
 FN(compact) {  // mask, coords, row_of, batch_offsets, count, stream
     return entry<6>(args, nargs, [](PyObject* const* a) {
         const at::Tensor& m = tensor(a[0]);
@@ -134,7 +162,7 @@ FN(compact) {  // mask, coords, row_of, batch_offsets, count, stream
         const auto* mask = static_cast<const uint8_t*>(dev(&m));
         I32 *c = ptr<I32>(a[1]), *r = ptr<I32>(a[2]), *o = ptr<I32>(a[3]), *n = ptr<I32>(a[4]);
         const hc_stream_t s = stream(a[5]);
-        return unlocked([&] { return F(mask, B, V, c, r, o, n, s); });
+        return unlocked([&] { return (lib.*F)(mask, B, V, c, r, o, n, s); });
     });
 }
 
@@ -151,7 +179,7 @@ FN(sparse_spiral_conv_fwd) {
         const float* b = ptr<float>(a[9]);
         const hc_stream_t s = stream(a[12]);
         return unlocked([&] {
-            return hc_sparse_spiral_conv_fwd(xp, (hc_layout)layout, dt, c, r, n, spp, B, V, L, ci, co,
+            return lib.hc_sparse_spiral_conv_fwd(xp, (hc_layout)layout, dt, c, r, n, spp, B, V, L, ci, co,
                                              Wp, b, (hc_act)act, y, s);
         });
     });
@@ -165,7 +193,7 @@ FN(conv_rulebook) {  // coords, row_of, count, spiral, B, V, x_layout, rulebook,
         const auto* spp = static_cast<I32*>(dev(&sp));
         const hc_stream_t s = stream(a[8]);
         return unlocked([&] {
-            return hc_conv_rulebook(c, r, n, spp, B, V, L, (hc_layout)layout, rb, s);
+            return lib.hc_conv_rulebook(c, r, n, spp, B, V, L, (hc_layout)layout, rb, s);
         });
     });
 }
@@ -181,7 +209,7 @@ FN(mask_compact_rulebook) {
             *rb = ptr<I32>(a[7]);
         const hc_stream_t s = stream(a[8]);
         return unlocked([&] {
-            return hc_mask_compact_rulebook(mask, B, V, spp, L, (hc_layout)layout, c, r, o, n, rb, s);
+            return lib.hc_mask_compact_rulebook(mask, B, V, spp, L, (hc_layout)layout, c, r, o, n, rb, s);
         });
     });
 }
@@ -204,9 +232,9 @@ FN(sparse_conv_rulebook_fwd) {
         const long long hint = hinted ? integer64(a[7]) : 0;
         const hc_stream_t s = stream(a[10]);
         return unlocked([&] {
-            return hinted ? hc_sparse_conv_rulebook_fwd_hint(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b,
+            return hinted ? lib.hc_sparse_conv_rulebook_fwd_hint(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b,
                                                              (hc_act)act, yp, c, B, V, op, hint, s)
-                          : hc_sparse_conv_rulebook_fwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b,
+                          : lib.hc_sparse_conv_rulebook_fwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b,
                                                         (hc_act)act, yp, c, B, V, op, s);
         });
     });
@@ -222,7 +250,7 @@ FN(sparse_linear_fwd) {  // x, count, W, bias, act, y, stream
         const float* b = ptr<float>(a[3]);
         const hc_stream_t s = stream(a[6]);
         return unlocked([&] {
-            return hc_sparse_linear_fwd(xp, dt, n, cap, ci, co, Wp, b, (hc_act)act, y, s);
+            return lib.hc_sparse_linear_fwd(xp, dt, n, cap, ci, co, Wp, b, (hc_act)act, y, s);
         });
     });
 }
@@ -239,7 +267,7 @@ FN(sparse_group_norm_fwd) {  // x, batch_offsets, G, eps, gamma, beta, act, y, s
         const float *ga = ptr<float>(a[4]), *be = ptr<float>(a[5]);
         const hc_stream_t s = stream(a[8]);
         return unlocked([&] {
-            return hc_sparse_group_norm_fwd(xp, dt, op, B, cap, C, G, eps, ga, be, (hc_act)act, y, s);
+            return lib.hc_sparse_group_norm_fwd(xp, dt, op, B, cap, C, G, eps, ga, be, (hc_act)act, y, s);
         });
     });
 }
@@ -260,7 +288,7 @@ FN(sparse_conv_gn_fwd) {
         const float *b = ptr<float>(a[4]), *ga = ptr<float>(a[9]), *be = ptr<float>(a[10]);
         const hc_stream_t s = stream(a[13]);
         return unlocked([&] {
-            return hc_sparse_conv_gn_fwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b, c, op, B, G, eps, ga,
+            return lib.hc_sparse_conv_gn_fwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, b, c, op, B, G, eps, ga,
                                          be, (hc_act)act, yp, s);
         });
     });
@@ -274,7 +302,7 @@ FN(conv_rulebook_transpose) {  // rulebook, count, x_rows, row_ptr, taps, stream
         const I32* n = ptr<I32>(a[1]);
         I32 *p = ptr<I32>(a[3]), *t = ptr<I32>(a[4]);
         const hc_stream_t s = stream(a[5]);
-        return unlocked([&] { return hc_conv_rulebook_transpose(rbp, n, cap, L, xr, p, t, s); });
+        return unlocked([&] { return lib.hc_conv_rulebook_transpose(rbp, n, cap, L, xr, p, t, s); });
     });
 }
 
@@ -291,7 +319,7 @@ FN(sparse_conv_rulebook_bwd) {
         float *dW = ptr<float>(a[10]), *db = ptr<float>(a[11]);
         const hc_stream_t s = stream(a[12]);
         return unlocked([&] {
-            return hc_sparse_conv_rulebook_bwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, y, dy,
+            return lib.hc_sparse_conv_rulebook_bwd(xp, dt, xr, rbp, n, cap, L, ci, co, Wp, y, dy,
                                                (hc_act)act, p, t, dx, dW, db, s);
         });
     });
@@ -306,7 +334,7 @@ FN(mask_score_update) {  // O, alpha_in, alpha_out, sim, stream
         const float* ai = ptr<float>(a[1]);
         float *ao = ptr<float>(a[2]), *sim = ptr<float>(a[3]);
         const hc_stream_t s = stream(a[4]);
-        return unlocked([&] { return hc_mask_score_update(Op, dt, K, N, D, ai, ao, sim, s); });
+        return unlocked([&] { return lib.hc_mask_score_update(Op, dt, K, N, D, ai, ao, sim, s); });
     });
 }
 
@@ -317,7 +345,7 @@ FN(mask_select_topk) {  // alpha, kappa, selected, stream
         const auto* ap = static_cast<float*>(dev(&al));
         I32* sel = ptr<I32>(a[2]);
         const hc_stream_t s = stream(a[3]);
-        return unlocked([&] { return hc_mask_select_topk(ap, K, kappa, sel, s); });
+        return unlocked([&] { return lib.hc_mask_select_topk(ap, K, kappa, sel, s); });
     });
 }
 
@@ -329,7 +357,7 @@ FN(kappa_masks) {  // masks, selected, B, out, stream
         const auto* sp = static_cast<I32*>(dev(&sel));
         uint8_t* out = ptr<uint8_t>(a[3]);
         const hc_stream_t s = stream(a[4]);
-        return unlocked([&] { return hc_kappa_masks(mp, K, V, sp, kappa, B, out, s); });
+        return unlocked([&] { return lib.hc_kappa_masks(mp, K, V, sp, kappa, B, out, s); });
     });
 }
 
@@ -342,7 +370,7 @@ FN(gather_rows) {  // x, coords, count, frames_per_sample, y, stream
         void *xp = dev(&x, true), *yp = dev(&y, true);
         const I32 *c = ptr<I32>(a[1]), *n = ptr<I32>(a[2]);
         const hc_stream_t s = stream(a[5]);
-        return unlocked([&] { return hc_gather_rows(xp, dt, B, V, C, c, n, cap, fps, yp, s); });
+        return unlocked([&] { return lib.hc_gather_rows(xp, dt, B, V, C, c, n, cap, fps, yp, s); });
     });
 }
 
@@ -354,7 +382,7 @@ FN(scatter_dense) {  // y, coords, row_of, count, B, V, zero_fill, out, stream
         void *yp = dev(&y), *out = ptr(a[7]);
         const I32 *c = ptr<I32>(a[1]), *r = ptr<I32>(a[2]), *n = ptr<I32>(a[3]);
         const hc_stream_t s = stream(a[8]);
-        return unlocked([&] { return hc_scatter_dense(yp, dt, c, r, n, B, V, C, zf, out, s); });
+        return unlocked([&] { return lib.hc_scatter_dense(yp, dt, c, r, n, B, V, C, zf, out, s); });
     });
 }
 
@@ -369,15 +397,37 @@ FN(spiral_conv_fwd) {  // x, spiral, W, bias, act, y, stream
         const float* b = ptr<float>(a[3]);
         const hc_stream_t s = stream(a[6]);
         return unlocked([&] {
-            return hc_spiral_conv_fwd(xp, dt, spp, B, V, L, ci, co, Wp, b, (hc_act)act, y, s);
+            return lib.hc_spiral_conv_fwd(xp, dt, spp, B, V, L, ci, co, Wp, b, (hc_act)act, y, s);
         });
     });
 }
 
 #define METHOD(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, nullptr}
+
+PyObject* bind(PyObject*, PyObject* arg) {  // the dlopen handle of libhc, as an int
+    void* handle = PyLong_AsVoidPtr(arg);
+    if (!handle) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "no library handle");
+        return nullptr;
+    }
+    Library l;
+#define LOOK_UP(f)                                                              \
+    l.f = reinterpret_cast<decltype(l.f)>(dlsym(handle, #f));                   \
+    if (!l.f) {                                                                 \
+        PyErr_SetString(PyExc_RuntimeError, "the library does not have " #f);   \
+        return nullptr;                                                         \
+    }
+    HC_CALLS(LOOK_UP)
+#undef LOOK_UP
+    lib = l;
+    bound = true;
+    Py_RETURN_NONE;
+}
+
 PyMethodDef methods[] = {
-    METHOD("hc_mask_compact", compact<hc_mask_compact>),
-    METHOD("hc_mask_compact_static", compact<hc_mask_compact_static>),
+    {"bind", bind, METH_O, nullptr},
+    METHOD("hc_mask_compact", compact<&Library::hc_mask_compact>),
+    METHOD("hc_mask_compact_static", compact<&Library::hc_mask_compact_static>),
     METHOD("hc_sparse_spiral_conv_fwd", sparse_spiral_conv_fwd),
     METHOD("hc_conv_rulebook", conv_rulebook),
     METHOD("hc_mask_compact_rulebook", mask_compact_rulebook),

@@ -11,7 +11,7 @@ The tensors are read and checked by a small extension module
 host time, more than most small layers take on the GPU; it costs 2.3 us here
 (the launch included).
 load_library() still hands out libhc itself through ctypes, for callers with
-raw pointers.
+raw pointers; the extension calls that same library, whatever its path.
 """
 from __future__ import annotations
 
@@ -119,6 +119,7 @@ def _load_native():
             spec = importlib.util.spec_from_file_location("_hc_native", NATIVE_PATH)
             module = importlib.util.module_from_spec(spec)
             spec.loader.exec_module(module)
+            module.bind(_lib._handle)  # the library that load_library() opened
             _native = module
         return _native
 
