@@ -20,6 +20,8 @@ import importlib.util
 import os
 import threading
 
+from . import build
+
 PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(PKG, "_build", "libhc.so")
 NATIVE_PATH = os.path.join(PKG, "_build", "_hc_native.so")
@@ -115,6 +117,9 @@ def _load_native():
             import torch  # noqa: F401  (the extension uses its libraries)
             if not os.path.exists(NATIVE_PATH):
                 raise RuntimeError(f"libhc's binding is not built ({NATIVE_PATH} missing): run "
+                                   "__graft_entry__.build()")
+            if not build.binding_matches():  # it would read tensors at wrong offsets
+                raise RuntimeError("libhc's binding was built for another torch or Python: run "
                                    "__graft_entry__.build()")
             spec = importlib.util.spec_from_file_location("_hc_native", NATIVE_PATH)
             module = importlib.util.module_from_spec(spec)
