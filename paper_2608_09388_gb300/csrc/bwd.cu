@@ -467,14 +467,24 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// A block takes kSortRows consecutive rows, whose entries are one slice of
-// taps, staged in shared memory in one coalesced copy. A thread per entry
-// counts the smaller entries of its row (about L of them; keys are unique) and
-// writes it at that place, so the work is even however few of the rows have
-// entries (5% of them in a dense input: a thread per row took twice as long).
-// A slice that does not fit is sorted row by row in place.
+// A block takes `per` consecutive rows (at most kSortRows), whose entries are
+// one slice of taps, staged in shared memory in one coalesced copy. A thread
+// per entry counts the smaller entries of its row (about L of them; keys are
+// unique) and writes it at that place, so the work is even however few of the
+// rows have entries (5% of them in a dense input: a thread per row took twice
+// as long). A slice has about L entries a row where every tap is present and
+// is not even, hence sort_rows: it fits kSortKeys with a quarter to spare (with
+// 256 rows at every L, the slices of 20 and more slots did not fit: 83.8k rows,
+// 24 slots, all present: 719 us, 72 us as it is). A slice that does not fit all the same (a few
+// rows with very many entries) is sorted row by row: up to 32 entries by a
+// warp, more by one of its lanes.
 constexpr int kSortRows = 256;
 constexpr int kSortKeys = 5120;
+
+constexpr int sort_rows(int L) {
+    return L <= kSortKeys * 4 / 5 / kSortRows ? kSortRows : kSortRows / 2;
+}
+static_assert(sort_rows(HC_MAX_SPIRAL) * HC_MAX_SPIRAL <= kSortKeys * 4 / 5, "a slice fits");
 
 __device__ __forceinline__ void insertion_sort(int32_t* taps, int a, int b) {
     for (int i = a + 1; i < b; ++i) {
@@ -488,8 +498,24 @@ __device__ __forceinline__ void insertion_sort(int32_t* taps, int a, int b) {
     }
 }
 
+// The warp sorts taps[a, b).
+__device__ __forceinline__ void sort_row(int32_t* taps, int a, int b) {
+    const int lane = threadIdx.x & 31, len = b - a;
+    if (len <= 1) return;
+    if (len <= 32) {
+        const int key = lane < len ? taps[a + lane] : 0x7fffffff;
+        int rank = 0;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) rank += __shfl_sync(0xffffffffu, key, k) < key;
+        if (lane < len) taps[a + rank] = key;
+    } else if (lane == 0) {
+        insertion_sort(taps, a, b);
+    }
+    __syncwarp();
+}
+
 __global__ void __launch_bounds__(kSortRows)
-    rb_sort_kernel(const int32_t* __restrict__ ptr, int x_rows, int32_t* __restrict__ taps) {
+    rb_sort_kernel(const int32_t* __restrict__ ptr, int x_rows, int per, int32_t* __restrict__ taps) {
     __shared__ int32_t s_keys[kSortKeys];
     __shared__ uint8_t s_row[kSortKeys];  // row (in the block) of an entry
     __shared__ int s_ptr[kSortRows + 1];
@@ -497,19 +523,19 @@ __global__ void __launch_bounds__(kSortRows)
     pdl_wait();
     pdl_trigger();
     const int t = threadIdx.x;
-    const long long r0 = (long long)blockIdx.x * kSortRows;
-    const int n = x_rows - r0 < kSortRows ? (int)(x_rows - r0) : kSortRows;
+    const long long r0 = (long long)blockIdx.x * per;
+    const int n = x_rows - r0 < per ? (int)(x_rows - r0) : per;
     if (t < n) s_ptr[t] = __ldg(ptr + r0 + t);
     if (t == 0) s_ptr[n] = __ldg(ptr + r0 + n);
     __syncthreads();
     const int base = s_ptr[0], len = s_ptr[n] - base;
-    const int a = t < n ? s_ptr[t] : 0, b = t < n ? s_ptr[t + 1] : 0;
     if (len > kSortKeys) {
-        if (b - a > 1) insertion_sort(taps, a, b);
+        for (int r = t >> 5; r < n; r += kSortRows / 32) sort_row(taps, s_ptr[r], s_ptr[r + 1]);
         return;
     }
     for (int i = t; i < len; i += kSortRows) s_keys[i] = taps[base + i];
-    for (int i = a - base; i < b - base; ++i) s_row[i] = (uint8_t)t;
+    if (t < n)
+        for (int i = s_ptr[t] - base; i < s_ptr[t + 1] - base; ++i) s_row[i] = (uint8_t)t;
     __syncthreads();
     for (int i = t; i < len; i += kSortRows) {
         const int key = s_keys[i], r = s_row[i];
@@ -1818,8 +1844,9 @@ hc_status launch_rulebook_transpose(const DeviceCtx* ctx, const int32_t* rb, con
     st = launch_pdl(rb_fill_kernel, grid, dim3(256), 0, s, "rb_fill_kernel", rb, count,
                     (long long)capacity, L, x_rows, (const int32_t*)ptr, (const int32_t*)place, taps);
     if (st != HC_OK) return st;
-    return launch_pdl(rb_sort_kernel, dim3((unsigned)((x_rows + kSortRows - 1) / kSortRows)),
-                      dim3(kSortRows), 0, s, "rb_sort_kernel", (const int32_t*)ptr, x_rows, taps);
+    const int per = sort_rows(L);
+    return launch_pdl(rb_sort_kernel, dim3((unsigned)(((long long)x_rows + per - 1) / per)),
+                      dim3(kSortRows), 0, s, "rb_sort_kernel", (const int32_t*)ptr, x_rows, per, taps);
 }
 
 hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s) {
