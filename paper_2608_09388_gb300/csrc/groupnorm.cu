@@ -735,6 +735,12 @@ __global__ void __launch_bounds__(kThreads, 4)
 // barrier. Rows past kClSlots per thread are read a second time instead. g is
 // the fewest CTAs that hold an average frame, or more where there would be
 // idle ones, chosen on the device from the frame table (the same in every CTA).
+// Frames of very different sizes are taken by size (gn_cluster_uneven): by the
+// average alone one frame of 10475 rows among 63 empty ones fell to 4 CTAs (48
+// us; 17-19 us as it is, 21 us by the row ranges; 8 such frames 70, 23 and 31 us;
+// every other frame 78, 61 and 66 us; 512 channels, one frame: 92, 24 and 27 us).
+// Telling them apart, behind the first copies, costs every call 0.5-1.5 us (64 x
+// 10475 94.7 -> 96.4 us).
 // Two CTAs share an SM, so that one's arithmetic overlaps the other's memory
 // accesses.
 // The issue slots bound it next to memory, hence the packed arithmetic and four
@@ -747,7 +753,8 @@ constexpr int kClCtas = 8;
 constexpr int kClThreads = 256;
 constexpr int kClSlots = 24;
 constexpr int kClGroup = 8;  // slots per cp.async group
-constexpr size_t kClSmem = (size_t)kClSlots * kClThreads * 16;
+constexpr int kClList = 512;  // frames listed at most
+constexpr size_t kClSlotBytes = (size_t)kClSlots * kClThreads * 16;
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
@@ -838,43 +845,68 @@ __device__ __forceinline__ void add_four(Stats& st, const Raw (&raw)[4]) {
     st.n = nn;
 }
 
-template <typename T, int ACT>
-__global__ void __launch_bounds__(kClThreads, 2)
-    gn_cluster_kernel(const T* x, const int32_t* __restrict__ offsets, int B, int C, int pc_max, int cpc,
-                      long long capacity, float eps, const float* __restrict__ gamma,
-                      const float* __restrict__ beta, T* y, unsigned* status) {
+struct ClShared {  // behind the slots
+    float red[kClThreads / 32][32][3];
+    float part[2][32][3];  // this CTA's sums of the unit, by round parity
+    float mu[32], inv[32];
+    int warp[kClThreads / 32];
+    int order[kClList];  // frames in the order they are taken
+};
+constexpr size_t kClSmem = kClSlotBytes + sizeof(ClShared);
+
+template <typename T>
+struct ClArgs {
+    const T* x;
+    const int32_t* offsets;
+    int B, C, pc_max, cpc;
+    float eps;
+    const float *gamma, *beta;
+    T* y;
+    long long o0, oB;  // the table's ends
+
+    // half-width parts where the slots of a cluster do not hold a frame of
+    // `rows` rows at full width
+    __device__ int held() const { return kClCtas * kClSlots * (kClThreads / pc_max); }
+    __device__ int part_chunks(long long rows) const {
+        return rows > held() && pc_max / 2 >= cpc && pc_max / 2 >= 4 ? pc_max / 2 : pc_max;
+    }
+    // CTAs of a unit, frames of `rows` rows on average
+    __device__ int ctas(long long frames, long long rows, int pc) const {
+        const long long units = frames * (C / (16 / (int)sizeof(T)) / pc);
+        int g = 1;
+        while (g < kClCtas &&
+               (rows > (long long)g * kClSlots * (kClThreads / pc) || units * g * 2 <= gridDim.x))
+            g *= 2;
+        return g;
+    }
+};
+
+// The frames from..to - 1 of the table (kListed: of the listed order), without
+// those above skip rows, in parts of pc chunks, g CTAs a unit, unit after unit
+// over the clusters. par: parity of the rounds so far. go_on() is asked behind
+// the first copies; without it nothing is done.
+template <typename T, int ACT, bool kListed, class GoOn>
+__device__ __forceinline__ void gn_cluster_run(const ClArgs<T>& a, int from, int to, int pc, int g,
+                                               int skip, int& par, GoOn&& go_on) {
     constexpr int VEC = 16 / (int)sizeof(T);
     using CK = Chunk<T, VEC>;
     using Raw = typename CK::Raw;
     constexpr int kWarps = kClThreads / 32;
     extern __shared__ __align__(16) uint8_t slots[];
-    __shared__ float s_red[kWarps][32][3];
-    __shared__ float s_part[2][32][3];  // this CTA's sums of the unit, by round parity
-    __shared__ float s_mu[32], s_inv[32];
+    ClShared& sh = *reinterpret_cast<ClShared*>(slots + kClSlotBytes);
+    const T* const x = a.x;
+    const int32_t* const __restrict__ offsets = a.offsets;
+    const float *const __restrict__ gamma = a.gamma, *const __restrict__ beta = a.beta;
+    T* const y = a.y;
+    const int C = a.C, cpc = a.cpc;
+    const float eps = a.eps;
+    const long long o0 = a.o0, oB = a.oB;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int rank = blockIdx.x % kClCtas, cluster = blockIdx.x / kClCtas;
     const int clusters = gridDim.x / kClCtas;
-    pdl_wait();
-    pdl_trigger();
-    const long long o0 = __ldg(offsets), oB = __ldg(offsets + B);
-    // frames must be in order (each CTA checks a share of the table)
-    for (long long i = (long long)blockIdx.x * kClThreads + t; i < B;
-         i += (long long)gridDim.x * kClThreads)
-        if (__ldg(offsets + i + 1) < __ldg(offsets + i)) report(status, kErrIndex);
-    if (o0 < 0 || oB < o0 || oB > capacity) {
-        if (t == 0 && blockIdx.x == 0) report(status, kErrIndex);
-        return;  // every CTA alike
-    }
-    // half-width parts where the slots of a cluster do not hold an average
-    // frame at full width
-    const long long avg = (oB - o0 + B - 1) / B;
-    int pc = pc_max;
-    if (avg > (long long)kClCtas * kClSlots * (kClThreads / pc) && pc / 2 >= cpc && pc / 2 >= 4) pc /= 2;
     const int parts = C / VEC / pc;
     const int rpp = kClThreads / pc;  // rows of a slot
-    const long long units = (long long)B * parts;
-    int g = 1;
-    while (g < kClCtas && (avg > (long long)g * kClSlots * rpp || units * g * 2 <= gridDim.x)) g *= 2;
+    const long long units = (long long)(to - from) * parts;
     const int per = kClCtas / g;  // units of a cluster at a time
     const int sub = rank / g, r = rank - sub * g;
     const long long rounds = (units + (long long)clusters * per - 1) / ((long long)clusters * per);
@@ -889,24 +921,25 @@ __global__ void __launch_bounds__(kClThreads, 2)
         int rows, col;
     };
     auto locate = [&](long long round) {
-        Share sh{0, 0, tc * VEC};
+        Share s{0, 0, tc * VEC};
         const long long u = (round * clusters + cluster) * per + sub;
-        if (round >= rounds || u >= units) return sh;
-        const int b = (int)(u / parts);
-        sh.col = ((int)(u - (long long)b * parts) * pc + tc) * VEC;
+        if (round >= rounds || u >= units) return s;
+        const int f = (int)(u / parts), b = kListed ? sh.order[from + f] : from + f;
+        s.col = ((int)(u - (long long)f * parts) * pc + tc) * VEC;
         const long long f0 = __ldg(offsets + b), f1 = __ldg(offsets + b + 1);
-        if (f0 < o0 || f1 < f0 || f1 > oB) return sh;  // reported above, or outside the span
-        const long long n = f1 - f0, s0 = f0 + n * r / g, s1 = f0 + n * (r + 1) / g;
-        sh.rows = (int)(s1 - s0) - tr;
-        sh.at = (s0 + tr) * C + sh.col;
-        return sh;
+        if (f0 < o0 || f1 < f0 || f1 > oB) return s;  // reported above, or outside the span
+        const long long n = f1 - f0, r0 = f0 + n * r / g, r1 = f0 + n * (r + 1) / g;
+        if (!kListed && n > skip) return s;
+        s.rows = (int)(r1 - r0) - tr;
+        s.at = (r0 + tr) * C + s.col;
+        return s;
     };
     const long long step = (long long)rpp * C;
-    auto copies = [&](const Share& sh, int i0, int i1) {
+    auto copies = [&](const Share& s, int i0, int i1) {
 #pragma unroll 4
         for (int i = i0; i < i1; ++i)
-            if (i * rpp < sh.rows)
-                cp_async_16(slot0 + (uint32_t)i * (kClThreads * 16u), x + sh.at + i * step, true);
+            if (i * rpp < s.rows)
+                cp_async_16(slot0 + (uint32_t)i * (kClThreads * 16u), x + s.at + i * step, true);
         cp_async_commit();
     };
     auto slot = [&](int i) {
@@ -915,8 +948,11 @@ __global__ void __launch_bounds__(kClThreads, 2)
 
     Share cur = locate(0);
     for (int i = 0; i < kClSlots; i += kClGroup) copies(cur, i, i + kClGroup);
-    for (long long round = 0; round < rounds; ++round) {
-        const int par = (int)(round & 1);
+    if (!go_on()) {
+        cp_async_wait_all();
+        return;
+    }
+    for (long long round = 0; round < rounds; ++round, par ^= 1) {
         // statistics
         Stats st;
         const int mine = cur.rows > 0 ? (cur.rows + rpp - 1) / rpp : 0;  // chunks of this thread
@@ -956,7 +992,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
         for (int o = 1; o < cpc; o <<= 1) merge_into_xor(st.n, st.mean, st.m2, o);
         for (int o = pc; o < 32; o <<= 1) merge_into_xor(st.n, st.mean, st.m2, o);
         if (lane < pc && lane % cpc == 0) {
-            float* e = s_red[warp][lane / cpc];
+            float* e = sh.red[warp][lane / cpc];
             e[0] = st.n, e[1] = st.mean, e[2] = st.m2;
         }
         __syncthreads();
@@ -964,27 +1000,27 @@ __global__ void __launch_bounds__(kClThreads, 2)
             float n = 0.f, mean = 0.f, m2 = 0.f;
 #pragma unroll
             for (int w = 0; w < kWarps; ++w)
-                merge_into(n, mean, m2, s_red[w][t][0], s_red[w][t][1], s_red[w][t][2]);
-            s_part[par][t][0] = n, s_part[par][t][1] = mean, s_part[par][t][2] = m2;
+                merge_into(n, mean, m2, sh.red[w][t][0], sh.red[w][t][1], sh.red[w][t][2]);
+            sh.part[par][t][0] = n, sh.part[par][t][1] = mean, sh.part[par][t][2] = m2;
         }
         if (g > 1) cluster_sync();
         else __syncthreads();
         for (int q = warp; q < groups; q += kWarps) {
             float n = 0.f, mean = 0.f, m2 = 0.f;
             if (lane < g) {
-                const uint32_t e = smem_u32(&s_part[par][q][0]);
+                const uint32_t e = smem_u32(&sh.part[par][q][0]);
                 n = ld_cluster(e, sub * g + lane);
                 mean = ld_cluster(e + 4u, sub * g + lane);
                 m2 = ld_cluster(e + 8u, sub * g + lane);
             }
             for (int o = 1; o < g; o <<= 1) merge_into_xor(n, mean, m2, o);
             if (lane == 0) {
-                s_mu[q] = mean;
-                s_inv[q] = 1.f / sqrtf(m2 / n + eps);
+                sh.mu[q] = mean;
+                sh.inv[q] = 1.f / sqrtf(m2 / n + eps);
             }
         }
         __syncthreads();
-        const float mu = s_mu[tc / cpc], inv = s_inv[tc / cpc];
+        const float mu = sh.mu[tc / cpc], inv = sh.inv[tc / cpc];
         const uint64_t off = pk(-mu, -mu);
         uint64_t sc[VEC / 2], be[VEC / 2];
 #pragma unroll
@@ -1033,7 +1069,143 @@ __global__ void __launch_bounds__(kClThreads, 2)
         }
         cur = next;
     }
-    if (g > 1) cluster_sync();  // no CTA leaves while another reads its sums
+    if (g > 1) cluster_sync();  // no CTA goes on or leaves while another reads its sums
+}
+
+// Uneven frames: those far above the average first (all, where whole clusters
+// take an average frame too), by whole clusters, then the others; both by
+// falling size, so that the clusters' shares are even, and without the empty
+// ones. Of many frames only the large ones are listed (the bound keeps them
+// few enough). Out of line: the even frames' code is what it is without this.
+template <typename T, int ACT>
+__device__ __noinline__ void gn_cluster_uneven(const ClArgs<T> a, int largest, int pc_avg, int g_avg) {
+    constexpr int kWarps = kClThreads / 32;
+    extern __shared__ __align__(16) uint8_t slots[];
+    ClShared& sh = *reinterpret_cast<ClShared*>(slots + kClSlotBytes);
+    int2* const frame = reinterpret_cast<int2*>(slots);  // (frame, rows); the slots are free yet
+    static_assert(kClList * sizeof(int2) <= kClSlotBytes, "the list fits");
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, B = a.B;
+    const long long total = a.oB - a.o0, avg = (total + B - 1) / B;
+    int large = 2 * avg < a.held() ? (int)(2 * avg) : a.held();
+    if (large < total / kClList) large = (int)(total / kClList);
+    const int fits = g_avg * kClSlots * (kClThreads / pc_avg);
+    if (large < fits) large = fits;
+    const bool all = B <= kClList;
+    if (all && g_avg == kClCtas) large = 0;
+    int listed = 0;
+    for (int i0 = 0; i0 < B; i0 += kClThreads) {
+        const int i = i0 + t;
+        const int n = i < B ? __ldg(a.offsets + i + 1) - __ldg(a.offsets + i) : 0;
+        const bool on = n > (all ? 0 : large);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        __syncthreads();  // sh.warp is free
+        if (lane == 0) sh.warp[warp] = __popc(m);
+        __syncthreads();
+        int at = listed + __popc(m & ((1u << lane) - 1u));
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            at += w < warp ? sh.warp[w] : 0;
+            listed += sh.warp[w];
+        }
+        if (on && at < kClList) frame[at] = make_int2(i, n);
+    }
+    if (listed > kClList) listed = kClList;  // a table out of order (reported)
+    __syncthreads();
+    int n_large = 0;
+    unsigned rest = 0;  // rows of the listed frames that are not large
+    for (int e = t; e < listed; e += kClThreads) {
+        const int2 f = frame[e];
+        int place = 0;
+        for (int j = 0; j < listed; ++j) {
+            const int n = frame[j].y;
+            place += n > f.y || (n == f.y && j < e);
+        }
+        sh.order[place] = f.x;
+        if (f.y > large) ++n_large;
+        else rest += (unsigned)f.y;
+    }
+    n_large = __reduce_add_sync(0xffffffffu, n_large);
+    rest = __reduce_add_sync(0xffffffffu, rest);
+    __syncthreads();
+    if (lane == 0) frame[warp] = make_int2(n_large, (int)rest);
+    __syncthreads();
+    n_large = 0, rest = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        n_large += frame[w].x;
+        rest += (unsigned)frame[w].y;
+    }
+    __syncthreads();  // the slots are the frames' from here on
+    int par = 0;
+    for (int part = 0; part < (all ? 2 : 1); ++part) {
+        const int from = part == 0 ? 0 : n_large, to = part == 0 ? n_large : listed;
+        const int rows = part == 0 ? largest : (int)(rest / (unsigned)(to > from ? to - from : 1));
+        const int pc = a.part_chunks(rows);
+        gn_cluster_run<T, ACT, true>(a, from, to, pc,
+                                     part == 0 ? kClCtas : a.ctas(to - from, rows, pc), 0, par,
+                                     [] { return true; });
+    }
+    if (!all)
+        gn_cluster_run<T, ACT, false>(a, 0, B, pc_avg, g_avg, large, par, [] { return true; });
+}
+
+template <typename T, int ACT>
+__global__ void __launch_bounds__(kClThreads, 2)
+    gn_cluster_kernel(const T* x, const int32_t* __restrict__ offsets, int B, int C, int pc_max, int cpc,
+                      long long capacity, float eps, const float* __restrict__ gamma,
+                      const float* __restrict__ beta, T* y, unsigned* status) {
+    extern __shared__ __align__(16) uint8_t slots[];
+    ClShared& sh = *reinterpret_cast<ClShared*>(slots + kClSlotBytes);
+    const int t = threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
+    const long long o0 = __ldg(offsets), oB = __ldg(offsets + B);
+    if (o0 < 0 || oB < o0 || oB > capacity) {
+        if (t == 0 && blockIdx.x == 0) report(status, kErrIndex);
+        return;  // every CTA alike
+    }
+    const ClArgs<T> a{x, offsets, B, C, pc_max, cpc, eps, gamma, beta, y, o0, oB};
+    const long long avg = (oB - o0 + B - 1) / B;
+    const int pc = a.part_chunks(avg), g = a.ctas(B, avg, pc);
+    // Uneven: some frame is more than a CTA holds, and the frames' mean square
+    // is well above their mean's (equal frames 1, sizes spread evenly from 0 on
+    // 1.33, every other frame empty 2), unless each unit has a cluster anyway.
+    // The same in every CTA.
+    int largest = 0;
+    bool uneven = false;
+    auto even = [&] {
+        float squares = 0.f;
+        bool ordered = true;
+#pragma unroll 4
+        for (int i = t; i < B; i += kClThreads) {
+            const int lo = __ldg(offsets + i), hi = __ldg(offsets + i + 1);
+            if (hi < lo) ordered = false;
+            const int n = hi < lo ? 0 : hi - lo;
+            largest = n > largest ? n : largest;
+            squares = fmaf((float)n, (float)n, squares);
+        }
+        if (!ordered) report(status, kErrIndex);  // frames must be in order
+        largest = __reduce_max_sync(0xffffffffu, largest);
+        for (int o = 16; o > 0; o >>= 1) squares += __shfl_xor_sync(0xffffffffu, squares, o);
+        if ((t & 31) == 0) {
+            sh.warp[t >> 5] = largest;
+            sh.mu[t >> 5] = squares;
+        }
+        __syncthreads();
+        squares = 0.f;
+#pragma unroll
+        for (int w = 0; w < kClThreads / 32; ++w) {
+            largest = sh.warp[w] > largest ? sh.warp[w] : largest;
+            squares += sh.mu[w];
+        }
+        const float mean = (float)(oB - o0) / (float)B;
+        uneven = largest > kClSlots * (kClThreads / pc_max) && squares > 1.6f * mean * mean * (float)B &&
+                 (g < kClCtas || (long long)B * (C / (16 / (int)sizeof(T)) / pc) * g > gridDim.x);
+        return !uneven;
+    };
+    int par = 0;
+    gn_cluster_run<T, ACT, false>(a, 0, B, pc, g, 0x7fffffff, par, even);
+    if (uneven) gn_cluster_uneven<T, ACT>(a, largest, pc, g);
 }
 
 long long fast_grid(const DeviceCtx* ctx, long long capacity) {
