@@ -306,6 +306,11 @@ __global__ void __launch_bounds__(C::THREADS, 1)
     }
 }
 
+// Calls that 64-row tiles cannot share out twice over the SMs.
+bool small_call(const DeviceCtx* ctx, const ConvArgs& a) {
+    return a.capacity <= 64ll * ctx->num_sms;
+}
+
 template <class C>
 hc_status launch_cfg(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
     static bool attr_set[64] = {};
@@ -329,23 +334,38 @@ hc_status launch_cfg(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-// The dense layer has no absent tap to skip. There the 64 x 64 tiles of
-// conv_simt.cu, eight blocks an SM, stay ahead where this kernel's rows come
-// element by element (45 -> 42 over 42k rows: 90 us there, 123 here) and where
-// its outputs are an odd number of 64-wide tiles above one (192 -> 192 over 5k
-// rows: 199 there, 223 here); elsewhere it is ahead (64 -> 64: 121 there, 114
-// here; 128 -> 128 over 21k rows: 230 there, 194 here).
-bool conv_f32_preferred(const ConvArgs& a) {
+// Where the 64 x 64 tiles of conv_simt.cu, eight blocks an SM, stay ahead. A
+// step is one slot, so with few input channels its barrier, gather and round
+// trip of the sums are for next to no multiply-adds, while those tiles take
+// several slots a step (41.9k rows, 9 slots, 3 -> 64: 44 us here, 22 there at
+// every tap present, 12.4 and 10.3 at 15%; 32 slots 129 and 30 us): below 16
+// channels, or 8 with the 128-output tiles (8 -> 128: 23 us here, 27 there at
+// half of the taps present).
+// The dense layer has no absent tap to skip besides, so it is not taken where
+// channels come element by element (45 -> 42 over 42k rows: 90 us there, 123
+// here), where an odd number of 64-wide tiles above one splits the outputs
+// (192 -> 192 over 5k rows: 199 and 223), and, with enough rows for the tall
+// tiles, where steps are mostly padding: 64-output tiles with steps of 64
+// channels (16 -> 64: 44 us there, 49 here; 36: 74 and 78; 56: 105 and 102; 72:
+// 134 and 141; 96: 173 and 171), 128-output ones with steps of 32 beyond the
+// first (32 -> 128: 110 and 107; 40: 134 and 148; 56: 180 and 181; 128: 390 and
+// 380; from 256 outputs on all are ahead here: 40: 260 and 252).
+bool conv_f32_preferred(const DeviceCtx* ctx, const ConvArgs& a) {
     const int tiles64 = (a.C_out + 63) / 64;
-    return a.mode != kDense || (a.C_in % 4 == 0 && (tiles64 == 1 || tiles64 % 2 == 0));
+    const bool wide = tiles64 % 2 == 0;
+    if (a.C_in < 8 || (a.C_in < 16 && !wide)) return false;
+    if (a.mode != kDense) return true;
+    if (a.C_in % 4 != 0 || a.C_in < 16 || (tiles64 > 1 && !wide)) return false;
+    if (small_call(ctx, a) || tiles64 >= 4) return true;
+    if (wide) return a.C_in <= 32 || 5 * a.C_in >= 4 * ((a.C_in + 31) / 32 * 32);
+    return a.C_in > 64 ? a.C_in % 64 == 0 || a.C_in % 64 >= 32 : a.C_in >= 48;
 }
 
 hc_status launch_conv_f32(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
-    // Calls that 64-row tiles cannot share out twice over the SMs are bound by
-    // round trips: the smaller table is resolved with fewer of them, and more
-    // steps are in flight. 16 input channels (a network's first layer) fit
+    // Small calls are bound by round trips: the smaller table is resolved with
+    // fewer of them, and more steps are in flight. 16 input channels (a network's first layer) fit
     // half a step.
-    const bool small = a.capacity <= 64ll * ctx->num_sms;
+    const bool small = small_call(ctx, a);
     const bool narrow = a.C_in <= 16;
     // 64-output tiles where 128-output ones would be half empty
     if ((a.C_out + 63) / 64 % 2 == 1) {

@@ -1,8 +1,8 @@
 // Spiral convolution / linear layer on CUDA cores (FFMA, fp32 accumulate) for
 // bf16 shapes the tensor-core kernel does not take (output channel counts that
-// are not a multiple of 8, misaligned rows), and for the fp32 dense layer at
-// some widths; other fp32 layers have a kernel of their own (conv_f32.cu). And
-// the narrow linear heads of both types.
+// are not a multiple of 8, misaligned rows), and for fp32 layers of few input
+// channels and the fp32 dense layer at some widths; other fp32 layers have a
+// kernel of their own (conv_f32.cu). And the narrow linear heads of both types.
 //
 // Each CTA owns a 64-row x 64-column output tile and walks K = L*C_in in
 // chunks of KC (128 when K <= 256, else 64): the A chunk is gathered through the per-tile table of source

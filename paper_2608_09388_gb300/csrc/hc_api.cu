@@ -114,7 +114,7 @@ hc_status dispatch_conv(const DeviceCtx* ctx, ConvArgs& a, hc_dtype dt, cudaStre
         return launch_conv_tc(ctx, a, s);
     }
     if (linear_head_supported(a, dt)) return launch_linear_head(ctx, a, dt, s);
-    if (dt == HC_F32 && conv_f32_preferred(a)) return launch_conv_f32(ctx, a, s);
+    if (dt == HC_F32 && conv_f32_preferred(ctx, a)) return launch_conv_f32(ctx, a, s);
     return launch_conv_simt(ctx, a, dt, s);
 }
 

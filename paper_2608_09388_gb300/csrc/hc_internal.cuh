@@ -114,7 +114,7 @@ struct ConvArgs {
 hc_status launch_compact(const DeviceCtx* ctx, const uint8_t* mask, int B, int V, int32_t* coords,
                          int32_t* row_of, int32_t* offsets, int32_t* count, cudaStream_t s);
 hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
-bool conv_f32_preferred(const ConvArgs& a);
+bool conv_f32_preferred(const DeviceCtx* ctx, const ConvArgs& a);
 hc_status launch_conv_f32(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
 bool linear_head_supported(const ConvArgs& a, hc_dtype dt);
 hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);

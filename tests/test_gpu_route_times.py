@@ -1,0 +1,55 @@
+"""Calls that a kernel made for larger or sparser ones must not slow down: each
+against a call of the same kind that takes the other kernel or is larger."""
+import pytest
+
+from paper_2608_09388_gb300 import hc
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_09388_gb300 import build
+    build.build()
+    hc.load_library()
+
+
+def us(f):
+    from _timing import device_us
+    return device_us(f)
+
+
+def count(n):
+    return torch.tensor([n], dtype=torch.int32, device="cuda")
+
+
+def neighbours(L, n):
+    g = torch.Generator("cuda").manual_seed(L)
+    return torch.stack([torch.randperm(n, generator=g, device="cuda") for _ in range(L)]).int()
+
+
+def conv_us(L, n, ci, co, dtype=torch.float32):
+    x, W = torch.randn((n, ci), device="cuda"), torch.randn((L * ci, co), device="cuda")
+    x, W = x.to(dtype), W.to(dtype)
+    y, rb, c = torch.empty((n, co), dtype=dtype, device="cuda"), neighbours(L, n), count(n)
+    return us(lambda: hc.hc_sparse_conv_rulebook_fwd(x, rb, c, W, None, hc.HC_ACT_ELU, y))
+
+
+def test_fp32_conv_of_few_channels():
+    """32 slots of 3 channels are 1.5 steps of 64, not 3.5 times 9 slots'."""
+    t9, t32 = conv_us(9, 41920, 3, 64), conv_us(32, 41920, 3, 64)
+    assert t32 < 2 * t9, (t9, t32)
+
+
+def test_fp32_dense_layer_of_few_channels():
+    """4 of 48 channels: not two fifths of the time."""
+    def dense(ci):
+        x = torch.randn((64, 655, ci), device="cuda")
+        W, sp = torch.randn((9 * ci, 64), device="cuda"), neighbours(9, 655).t().contiguous()
+        y = torch.empty((64, 655, 64), device="cuda")
+        return us(lambda: hc.hc_spiral_conv_fwd(x, sp, W, None, hc.HC_ACT_ELU, y))
+    few, many = dense(4), dense(48)
+    assert few < 0.31 * many, (few, many)
