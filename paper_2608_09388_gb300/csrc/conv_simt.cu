@@ -325,6 +325,22 @@ bool linear_head_supported(const ConvArgs& a, hc_dtype dt) {
            a.C_in * head_wpitch(a.C_out) <= kHeadMaxWFloats;
 }
 
+// Of those, the ones the 64 x 64 tiles serve better. A thread has a row's half
+// of the outputs, C_in channels of some groups of four one after the other; as
+// long as every SM has at most one 64-row tile, those tiles' 256 threads a tile
+// share that chain out further (655 rows, bf16 64 -> 60: 13.7 us there, 19.7
+// here; 128 -> 20: 15.4 and 19.5; 64 -> 28: 13.5 and 13.3; fp32 128 -> 16: 10.5
+// and 16.5; 64 -> 16: 8.7 and 9.8; 16 -> 16: 7.8 and 5.0), bf16 heads of more
+// than 48 outputs up to two tiles an SM (19k rows, 64 -> 60: 16.4 and 20.1; 64
+// -> 42: 16.4 and 17.0; 21k rows 27.7 and 21.9).
+bool linear_head_on_tiles(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt) {
+    const int groups = (head_wpitch(a.C_out) / kHeadGroup + 1) / 2;  // of a thread
+    const int chain = a.C_in * groups;
+    const bool f32 = dt == HC_F32;
+    const long long tiles = !f32 && a.C_out > 48 ? 2 : 1;
+    return (f32 ? chain >= 128 : chain > 256) && a.capacity <= 64 * tiles * ctx->num_sms;
+}
+
 hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s) {
     return dt == HC_F32 ? launch_head_typed<float>(ctx, a, s)
                         : launch_head_typed<__nv_bfloat16>(ctx, a, s);

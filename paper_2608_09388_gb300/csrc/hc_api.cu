@@ -113,7 +113,9 @@ hc_status dispatch_conv(const DeviceCtx* ctx, ConvArgs& a, hc_dtype dt, cudaStre
         }
         return launch_conv_tc(ctx, a, s);
     }
-    if (linear_head_supported(a, dt)) return launch_linear_head(ctx, a, dt, s);
+    if (linear_head_supported(a, dt))
+        return linear_head_on_tiles(ctx, a, dt) ? launch_conv_simt(ctx, a, dt, s)
+                                                : launch_linear_head(ctx, a, dt, s);
     if (dt == HC_F32 && conv_f32_preferred(ctx, a)) return launch_conv_f32(ctx, a, s);
     return launch_conv_simt(ctx, a, dt, s);
 }

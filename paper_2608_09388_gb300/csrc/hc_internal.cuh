@@ -117,6 +117,7 @@ hc_status launch_conv_simt(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt,
 bool conv_f32_preferred(const DeviceCtx* ctx, const ConvArgs& a);
 hc_status launch_conv_f32(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
 bool linear_head_supported(const ConvArgs& a, hc_dtype dt);
+bool linear_head_on_tiles(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt);
 hc_status launch_linear_head(const DeviceCtx* ctx, const ConvArgs& a, hc_dtype dt, cudaStream_t s);
 hc_status launch_conv_tc(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s);
 bool conv_tc_supported(const ConvArgs& a, hc_dtype dt);

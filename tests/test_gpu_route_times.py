@@ -53,3 +53,20 @@ def test_fp32_dense_layer_of_few_channels():
         return us(lambda: hc.hc_spiral_conv_fwd(x, sp, W, None, hc.HC_ACT_ELU, y))
     few, many = dense(4), dense(48)
     assert few < 0.31 * many, (few, many)
+
+
+def head_us(n, ci, co, dtype):
+    x, W = torch.randn((n, ci), device="cuda").to(dtype), torch.randn((ci, co), device="cuda").to(dtype)
+    y, c = torch.empty((n, co), dtype=dtype, device="cuda"), count(n)
+    return us(lambda: hc.hc_sparse_linear_fwd(x, c, W, None, hc.HC_ACT_NONE, y))
+
+
+def test_small_linear_heads():
+    """655 rows: a bf16 head of 60 outputs takes no longer than a one-slot conv of
+    as many channels, which takes the 64 x 64 tiles (1.4 times as long on the
+    narrow-head kernel); an fp32 head of 16 outputs no longer than one of 3 (1.5
+    times)."""
+    head, tiles = head_us(655, 64, 60, torch.bfloat16), conv_us(1, 655, 64, 60, torch.bfloat16)
+    assert head < 1.2 * tiles, (head, tiles)
+    many, few = (head_us(655, 128, co, torch.float32) for co in (16, 3))
+    assert many < 1.2 * few, (many, few)
