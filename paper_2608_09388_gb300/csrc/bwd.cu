@@ -1273,7 +1273,7 @@ struct TapCfg {
     static constexpr int kStageBytes = kABytes + BN * 128;
     static constexpr int kStages = BN == 64 ? 8 : 6;
     static constexpr uint32_t kTmemCols = 2 * BN;
-    static constexpr int kBars = 2 * kStages + 5;
+    static constexpr int kBars = 3 * kStages + 5;
     static constexpr int kMisc = kStages * kStageBytes;
     static constexpr int kEpi = kMisc + (8 * kBars + 16 + 2 * 33 * 4 + 127) / 128 * 128;
     static constexpr size_t kSmem = 1024 + kEpi + 8 * 2048;
@@ -1325,9 +1325,10 @@ __global__ void __launch_bounds__(kTapThreads, 1)
     const uint32_t sBar = base + C::kMisc;
     auto full_bar = [&](int s) { return sBar + 8u * s; };
     auto empty_bar = [&](int s) { return sBar + 8u * (kStages + s); };
-    auto tfull_bar = [&](int i) { return sBar + 8u * (2 * kStages + i); };
-    auto tempty_bar = [&](int i) { return sBar + 8u * (2 * kStages + 2 + i); };
-    const uint32_t fin_bar = sBar + 8u * (2 * kStages + 4);
+    auto wfull_bar = [&](int s) { return sBar + 8u * (2 * kStages + s); };
+    auto tfull_bar = [&](int i) { return sBar + 8u * (3 * kStages + i); };
+    auto tempty_bar = [&](int i) { return sBar + 8u * (3 * kStages + 2 + i); };
+    const uint32_t fin_bar = sBar + 8u * (3 * kStages + 4);
     uint8_t* const misc = base_ptr + C::kMisc + 8 * C::kBars;
     volatile uint32_t* const tmem_holder = reinterpret_cast<volatile uint32_t*>(misc);
     volatile int* const abort_flag = reinterpret_cast<volatile int*>(misc + 4);
@@ -1337,7 +1338,8 @@ __global__ void __launch_bounds__(kTapThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(full_bar(s), kProducerWarps * 32 + 1);
+            mbar_init(full_bar(s), kProducerWarps * 32);
+            mbar_init(wfull_bar(s), 1);
             mbar_init(empty_bar(s), 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -1437,9 +1439,9 @@ __global__ void __launch_bounds__(kTapThreads, 1)
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(full_bar(st), BN * 128);
+                    mbar_arrive_expect_tx(wfull_bar(st), BN * 128);
                     tma_load_2d(base + st * C::kStageBytes + C::kABytes, &tmap_w, kb * 64,
-                                l * a.C_in + c0, full_bar(st));
+                                l * a.C_in + c0, wfull_bar(st));
                     ++it;
                     if (++st == kStages) {
                         st = 0;
@@ -1447,9 +1449,12 @@ __global__ void __launch_bounds__(kTapThreads, 1)
                     }
                 }
             }
-            if (!ok)  // copies already issued land before the CTA exits
+            // copies already issued land before the CTA exits; their barriers
+            // count nothing else (with the gather's arrivals, which an unwinding
+            // producer does not make, each would be waited for to the limit)
+            if (!ok)
                 for (long long j = it > kStages ? it - kStages : 0; j < it; ++j)
-                    mbar_wait_drain(full_bar((int)(j % kStages)), (uint32_t)((j / kStages) & 1),
+                    mbar_wait_drain(wfull_bar((int)(j % kStages)), (uint32_t)((j / kStages) & 1),
                                     a.status);
         }
         __syncwarp();
@@ -1465,7 +1470,8 @@ __global__ void __launch_bounds__(kTapThreads, 1)
                     break;
                 tc_fence_after();
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(full_bar(st), ph, abort_flag, a.status)) {
+                    if (!mbar_wait(full_bar(st), ph, abort_flag, a.status) ||
+                        !mbar_wait(wfull_bar(st), ph, abort_flag, a.status)) {
                         ok = false;
                         break;
                     }
