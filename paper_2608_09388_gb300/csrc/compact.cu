@@ -415,15 +415,14 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
     // the first tap entries of this thread (item i: slot l = i / nact,
     // active vertex k = i % nact of the portion)
     const int items = nact * L;
-    int u_pre[kMapPre];
+    int u_pre[kMapPre], l_pre[kMapPre], k_pre[kMapPre];
 #pragma unroll
     for (int q = 0; q < kMapPre; ++q) {
         const int i = tid + q * kMapThreads;
         u_pre[q] = -1;
         if (i < items) {
-            int k;
-            const int l = (int)div32(i, nact, k);
-            u_pre[q] = __ldg(a.spiral + (long long)(v0 + act_v[k]) * L + l);
+            l_pre[q] = (int)div32(i, nact, k_pre[q]);
+            u_pre[q] = __ldg(a.spiral + (long long)(v0 + act_v[k_pre[q]]) * L + l_pre[q]);
         }
     }
 
@@ -453,7 +452,10 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
     unsigned err = 0;
     // the prefetched entries, then batches of kMapPre in flight (one by one a
     // portion with more entries paid a round trip for each: the headline layer
-    // 22.5 -> 21.6 us in graph replays; batches of 8: 21.8)
+    // 22.5 -> 21.6 us in graph replays; batches of 8: 21.8). Slot and vertex stay
+    // in registers from the load to the use: divided out a second time, masks
+    // with most vertices active lost more than the batches gave (32 x 10475, 12
+    // slots, all active 25.8 us; one by one 25.1; 23.9 as it is).
     for (int i0 = tid; i0 < items; i0 += kMapPre * kMapThreads) {
         if (i0 != tid) {
 #pragma unroll
@@ -461,9 +463,8 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
                 const int i = i0 + q * kMapThreads;
                 u_pre[q] = -1;
                 if (i < items) {
-                    int k;
-                    const int l = (int)div32(i, nact, k);
-                    u_pre[q] = __ldg(a.spiral + (long long)(v0 + act_v[k]) * L + l);
+                    l_pre[q] = (int)div32(i, nact, k_pre[q]);
+                    u_pre[q] = __ldg(a.spiral + (long long)(v0 + act_v[k_pre[q]]) * L + l_pre[q]);
                 }
             }
         }
@@ -471,8 +472,6 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
         for (int q = 0; q < kMapPre; ++q) {
             const int i = i0 + q * kMapThreads;
             if (i >= items) break;
-            int k;
-            const int l = (int)div32(i, nact, k);
             const int u = u_pre[q];
             int e = -1;
             if (u < -1 || u >= V) {
@@ -482,7 +481,7 @@ __global__ void __launch_bounds__(kMapThreads) compact_map_kernel(const MapArgs 
                 const int r = rank_of(u, hit);
                 if (hit) e = a.x_layout == HC_LAYOUT_DENSE ? (int)(fb + u) : off + r;
             }
-            a.rulebook[(long long)l * a.n + n0 + k] = e;
+            a.rulebook[(long long)l_pre[q] * a.n + n0 + k_pre[q]] = e;
         }
     }
     if (a.row_of)
