@@ -176,8 +176,9 @@ hc_status hc_conv_rulebook(const int32_t* coords, const int32_t* row_of, const i
 /*
  * hc_mask_compact_rulebook -- hc_mask_compact followed by hc_conv_rulebook on
  * its output (Eq. 2 and the Eq. 4 indexing matrix), in two kernels when
- * V <= 65535: a count pass (none for masks of up to 16 KB), then one pass
- * per (frame, block of 1024 vertices) that ranks the frame's mask bytes in shared memory and writes
+ * V <= 65535: a count pass (none for masks of up to 16 KB in few frames),
+ * then one pass per (frame, block of 1024 vertices) that ranks the frame's
+ * mask bytes in shared memory and writes
  * coords, row_of, batch_offsets, count and the rulebook columns of its
  * active vertices, every tap lookup answered from shared memory. Larger
  * frames run the two operations' own kernels. The results are identical to

@@ -522,8 +522,11 @@ hc_status launch_compact_map(const DeviceCtx* ctx, const uint8_t* mask, int B, i
     // Small masks need no count pass: every CTA counts the bytes before its
     // frame itself, at most one batch of loads a thread (one frame of 655: the
     // call 7.1 us against 10.5 with the count pass; 126 KB of masks that way
-    // took 21 us against 9.7).
-    const bool alone = n <= kMapAloneBytes;
+    // took 21 us against 9.7). So long as that is one wave: with more CTAs each
+    // of them pays for it (256 frames of 64: 4.3 us either way; 512 of 32: 5.8 us
+    // against 5.4; 16384 of one vertex: 83 against 70).
+    const long long ctas = (long long)B * ((V + kMapPortion - 1) / kMapPortion);
+    const bool alone = n <= kMapAloneBytes && ctas <= 2ll * ctx->num_sms;
     int32_t* tile_counts = nullptr;
     int prescanned = 0;
     if (!alone) {

@@ -70,3 +70,16 @@ def test_small_linear_heads():
     assert head < 1.2 * tiles, (head, tiles)
     many, few = (head_us(655, 128, co, torch.float32) for co in (16, 3))
     assert many < 1.2 * few, (many, few)
+
+
+def test_mapping_of_many_small_frames():
+    """16 KB of masks in one-vertex frames: a wave of CTAs that each count the whole
+    mask takes a fifth longer than the count pass, which one byte more brings."""
+    def mapping(B):
+        i32 = dict(dtype=torch.int32, device="cuda")
+        mask = (torch.arange(B, device="cuda") % 2).to(torch.uint8).view(B, 1)
+        spiral = torch.zeros((1, 1), **i32)
+        out = [torch.empty(s, **i32) for s in ((B, 2), (B, 1), (B + 1,), (1,), (1, B))]
+        return us(lambda: hc.hc_mask_compact_rulebook(mask, spiral, hc.HC_LAYOUT_DENSE, *out))
+    below, above = mapping(16384), mapping(16400)
+    assert below < 1.08 * above, (below, above)
