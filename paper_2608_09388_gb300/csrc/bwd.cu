@@ -21,6 +21,7 @@
 //                       per slot; tap GEMM: P[e] = dz[n] W_l^T for the e-th
 //                       tap (n, l) of the mapping; seg_sum: every input row
 //                       sums its own, consecutive rows of P, in (n, l) order.
+//                       With few channels P is over all (row, slot) pairs.
 // The transposed mapping itself: rb_* kernels (counts, exclusive scan, fill,
 // per-row sort).
 #include <cuda.h>
@@ -86,7 +87,7 @@ __host__ __device__ inline long long unit_rows(long long rows) {
 }
 
 struct PrepArgs {
-    int act_blocks, unit_blocks, hist_blocks;  // unit_blocks / hist_blocks: 0 = not wanted
+    int act_blocks, unit_blocks, hist_blocks, w_blocks;  // 0 = not wanted, but act_blocks
     const int32_t* rb;
     int L, x_rows;
     int32_t* unit_cnt;
@@ -94,6 +95,9 @@ struct PrepArgs {
     const int32_t* row_ptr;
     const int32_t* taps;
     int32_t* hist;
+    const void* W;  // copy_w
+    void* w_out;
+    int C_in, Cp, Cz;
     unsigned* status;
 };
 
@@ -169,7 +173,48 @@ __device__ void count_taps(const PrepArgs& p, const int32_t* count, long long ca
     if ((int)threadIdx.x < p.L) p.hist[b * p.L + threadIdx.x] = s_hist[threadIdx.x];
 }
 
+// W as the products of dgrad read it, by further blocks of the dz launch (a
+// launch of its own cost 1.5 us): over all pairs (Cp > 0), W^T [Cz][L * Cp]
+// with zeros where c >= C_in or o >= C_out, a 32 x 32 piece a block; else rows
+// of Cz columns, 1024 entries a block.
+template <typename T>
+__device__ void copy_w(const PrepArgs& p, int b, int C_out) {
+    __shared__ T tile[32][33];
+    const T* __restrict__ W = static_cast<const T*>(p.W);
+    T* __restrict__ out = static_cast<T*>(p.w_out);
+    if (p.Cp == 0) {
+        const long long n = (long long)p.L * p.C_in * p.Cz;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long i = b * 1024ll + q * 256 + threadIdx.x;
+            if (i >= n) break;
+            int o;
+            const long long m = div32(i, p.Cz, o);
+            out[i] = o < C_out ? W[m * C_out + o] : from_f<T>(0.f);
+        }
+        return;
+    }
+    const int K = p.L * p.Cp, kb = (K + 31) / 32;
+    const int k0 = b % kb * 32, o0 = b / kb * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int k = k0 + i, l = k / p.Cp, c = k - l * p.Cp, o = o0 + tx;
+        tile[i][tx] = k < K && c < p.C_in && o < C_out
+                          ? W[((long long)l * p.C_in + c) * C_out + o]
+                          : from_f<T>(0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int o = o0 + i, k = k0 + tx;
+        if (k < K && o < p.Cz) out[(long long)o * K + k] = tile[tx][i];
+    }
+}
+
 // ---------------------------------------------------------------- dz, dbias
+// Rows of dz have `pitch` columns: C_out, or with zeros behind them up to a
+// whole number of 16-byte chunks.
 // Block (64, 4): thread (tx, ty) takes columns g*64 + tx of rows r0 + ty +
 // 4 i of the block's row chunks (chunks blockIdx.x, + prep.act_blocks, ...); the
 // four row lanes' sums meet in shared memory and the block writes one
@@ -179,7 +224,7 @@ constexpr int kActRowsPerBlock = 16;
 template <typename T>
 __global__ void __launch_bounds__(256)
     act_bwd_kernel(const T* __restrict__ y, const T* __restrict__ dy, const int32_t* count,
-                   long long capacity, int C_out, int act, T* __restrict__ dz,
+                   long long capacity, int C_out, int act, T* __restrict__ dz, int pitch,
                    float* __restrict__ bpart, const PrepArgs prep, unsigned* status) {
     __shared__ float red[4][64];
     pdl_wait();
@@ -188,13 +233,18 @@ __global__ void __launch_bounds__(256)
         count_taps(prep, count, capacity);
         return;
     }
-    const int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
+    int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
+    if (block < prep.w_blocks) {
+        copy_w<T>(prep, block, C_out);
+        return;
+    }
+    block -= prep.w_blocks;
     const long long rows = clamp_rows(count, capacity, status);
     const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     for (int g0 = 0; g0 < C_out; g0 += 64) {
         const int o = g0 + tx;
         float sum = 0.f;
-        if (o < C_out)
+        if (o < pitch)
             for (long long r0 = (long long)block * kActRowsPerBlock; r0 < rows;
                  r0 += (long long)prep.act_blocks * kActRowsPerBlock) {
                 const long long r1 = r0 + kActRowsPerBlock < rows ? r0 + kActRowsPerBlock : rows;
@@ -204,8 +254,9 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const long long r = rb0 + 4 * i;
-                        yv[i] = r < r1 ? to_f(y[r * C_out + o]) : 0.f;
-                        gv[i] = r < r1 ? to_f(dy[r * C_out + o]) : 0.f;
+                        const bool in = r < r1 && o < C_out;
+                        yv[i] = in ? to_f(y[r * C_out + o]) : 0.f;
+                        gv[i] = in ? to_f(dy[r * C_out + o]) : 0.f;
                     }
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -215,7 +266,7 @@ __global__ void __launch_bounds__(256)
                         if (act == HC_ACT_ELU) d = yv[i] > 0.f ? 1.f : yv[i] + 1.f;
                         else if (act == HC_ACT_RELU) d = yv[i] > 0.f ? 1.f : 0.f;
                         const float v = gv[i] * d;
-                        dz[r * C_out + o] = from_f<T>(v);
+                        dz[r * pitch + o] = from_f<T>(v);  // columns past C_out: zeros
                         sum += v;
                     }
                 }
@@ -238,7 +289,7 @@ constexpr int kActVecItems = 1024;
 template <typename T>
 __global__ void __launch_bounds__(256)
     act_bwd_vec_kernel(const T* __restrict__ y, const T* __restrict__ dy, const int32_t* count,
-                       long long capacity, int C_out, int act, T* __restrict__ dz,
+                       long long capacity, int C_out, int act, T* __restrict__ dz, int,
                        float* __restrict__ bpart, const PrepArgs prep, unsigned* status) {
     constexpr int VEC = 16 / sizeof(T);
     constexpr int kPer = kActVecItems / 256;
@@ -249,7 +300,12 @@ __global__ void __launch_bounds__(256)
         count_taps(prep, count, capacity);
         return;
     }
-    const int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
+    int block = (int)blockIdx.x - prep.unit_blocks - prep.hist_blocks;
+    if (block < prep.w_blocks) {
+        copy_w<T>(prep, block, C_out);
+        return;
+    }
+    block -= prep.w_blocks;
     const long long rows = clamp_rows(count, capacity, status);
     const int t = threadIdx.x;
     const int cpr = C_out / VEC, lanes = 256 / cpr;
@@ -565,6 +621,7 @@ struct WgradArgs {
     const void* dz;
     long long capacity;
     int L, C_in, C_out;
+    int z_pitch;                 // columns of a row of dz
     int c_tiles, o_tiles, G;     // grid: G x (c_tiles * o_tiles)
     const int32_t* unit_cnt;     // [L][kUnits]
     const int2* unit_list;       // [L][capacity]
@@ -1008,7 +1065,7 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
                 for (int i = 0; i < 8; ++i) {
                     const int k = k0 + (t >> 7) + 2 * i;
                     const int n = k < want ? s_n[k] : -1;
-                    zv[i] = n >= 0 && o_ok ? to_f(dz[(long long)n * a.C_out + o]) : 0.f;
+                    zv[i] = n >= 0 && o_ok ? to_f(dz[(long long)n * a.z_pitch + o]) : 0.f;
                 }
             };
             fetch(0);
@@ -1567,7 +1624,7 @@ __global__ void __launch_bounds__(kTapThreads, 1)
     }
 }
 
-// CUDA cores: 128 listed taps x 64 channels per item, 8 x 4 per thread over
+// CUDA cores (fp32): 128 listed taps x 64 channels per item, 8 x 4 per thread over
 // chunks of 32 of C_out, the next chunk in registers while one is multiplied.
 // Both operands' rows are contiguous along C_out and are turned round on their
 // way into shared memory: a warp loads 8 values of 4 rows at a time, which are
@@ -1577,20 +1634,6 @@ __global__ void __launch_bounds__(kTapThreads, 1)
 // 128, 24% of the taps present).
 constexpr int kTgBM = 128, kTgBN = 64, kTgBK = 32;
 
-template <typename T>
-__device__ __forceinline__ void store4(T* dst, const float* v);
-template <>
-__device__ __forceinline__ void store4<float>(float* dst, const float* v) {
-    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-}
-template <>
-__device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* dst, const float* v) {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-    *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&a),
-                                                *reinterpret_cast<const uint32_t*>(&b));
-}
-
-template <typename T>
 __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs a) {
     __shared__ __align__(16) float As[kTgBK][kTgBM + 4];
     __shared__ __align__(16) float Bs[kTgBK][kTgBN + 4];
@@ -1599,9 +1642,9 @@ __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs
     pdl_trigger();
     if (threadIdx.x < 32) slot_tiles<kTgBM>(a.slot_off, a.L, s_off, s_tile);
     __syncthreads();
-    const T* __restrict__ dz = static_cast<const T*>(a.dz);
-    const T* __restrict__ W = static_cast<const T*>(a.W);
-    T* __restrict__ P = static_cast<T*>(a.P);
+    const float* __restrict__ dz = static_cast<const float*>(a.dz);
+    const float* __restrict__ W = static_cast<const float*>(a.W);
+    float* __restrict__ P = static_cast<float*>(a.P);
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     // loads: k = kl + 8 j; taps ra + 4 i, channels rb + 4 i
     const int kl = t & 7, ra = (t >> 5) * 16 + ((t >> 3) & 3), rb = (t >> 5) * 8 + ((t >> 3) & 3);
@@ -1637,9 +1680,9 @@ __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs
                 const int k = k0 + kl + 8 * j;
                 const bool in = k < a.C_out;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) av[i][j] = in && za[i] >= 0 ? to_f(dz[za[i] + k]) : 0.f;
+                for (int i = 0; i < 4; ++i) av[i][j] = in && za[i] >= 0 ? dz[za[i] + k] : 0.f;
 #pragma unroll
-                for (int i = 0; i < 2; ++i) bv[i][j] = in && wb[i] >= 0 ? to_f(W[wb[i] + k]) : 0.f;
+                for (int i = 0; i < 2; ++i) bv[i][j] = in && wb[i] >= 0 ? W[wb[i] + k] : 0.f;
             }
         };
         fetch(0);
@@ -1673,7 +1716,8 @@ __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const long long e = s_e[ty * 8 + i];
-                if (e >= 0) store4<T>(P + e * a.Cp + c, acc[i]);
+                if (e >= 0) *reinterpret_cast<float4*>(P + e * a.Cp + c) =
+                    make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
             }
         __syncthreads();  // s_e is free
     }
@@ -1691,10 +1735,13 @@ __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs
 // row whose range leaves the table is reported and becomes zeros.
 constexpr int kSegRows = 128;
 
-template <typename T>
+// kKeys: P has a row per key n*L + l (the product over all pairs), and e's row
+// is that of taps[e]; keys that no row has are reported and skipped.
+template <typename T, bool kKeys>
 __global__ void __launch_bounds__(256, 6)
-    seg_sum_kernel(const T* __restrict__ P, const int32_t* __restrict__ ptr, int x_rows, int C_in,
-                   int Cp, long long capL, T* __restrict__ dx, int vec_ok, unsigned* status) {
+    seg_sum_kernel(const T* __restrict__ P, const int32_t* __restrict__ ptr,
+                   const int32_t* __restrict__ taps, int x_rows, int C_in, int Cp, long long capL,
+                   T* __restrict__ dx, int vec_ok, unsigned* status) {
     constexpr int VEC = 16 / (int)sizeof(T);
     __shared__ int32_t s_ptr[kSegRows + 1];
     __shared__ uint16_t s_busy[kSegRows];
@@ -1756,13 +1803,22 @@ __global__ void __launch_bounds__(256, 6)
         for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
         for (int e = s_ptr[i]; e < e1; e += 4) {
             uint4 v[4];
+            bool use[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                use[q] = e + q < e1;
+                if (!kKeys) {
+                    if (use[q]) v[q] = ld_hint(P + (long long)(e + q) * Cp + col, let_go);
+                } else if (use[q]) {
+                    const int key = __ldg(taps + e + q);
+                    use[q] = key >= 0 && key < capL;
+                    if (use[q]) v[q] = ld_hint(P + (long long)key * Cp + col, let_go);
+                    else report(status, kErrIndex);
+                }
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (e + q < e1)
-                    v[q] = ld_hint(P + (long long)(e + q) * Cp + col, let_go);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (e + q < e1) {
+                if (kKeys ? use[q] : e + q < e1) {
                     const T* p = reinterpret_cast<const T*>(&v[q]);
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) acc[k] += to_f(p[k]);
@@ -1805,13 +1861,25 @@ hc_status launch_tap_gemm_tc(const DeviceCtx* ctx, const TapGemmArgs& g, cudaStr
                       TapCfg<BN>::kSmem, s, "tap_gemm_tc_kernel", g, tw);
 }
 
+// dx with few input channels: the product over all (row, slot) pairs, absent ones
+// too, as one linear layer dz W^T (rows of dz and slots of W padded to whole
+// chunks), whose rows seg_sum reads by key. A tile of the tap product has 64
+// channels of one slot, mostly padding here, and reads a row of dz for every tap
+// of it. 41.9k rows (mask full) or 4.9k (12%), 9 slots, dx alone, tap product and
+// this: bf16 16 -> 64 46 and 32 us, 14.6 and 12.4; 32 -> 64 46.7 and 35, 15.0 and
+// 13.0 (64 -> 64: 53 and 58); fp32 3 -> 64 97 and 35, 16.9 and 13.8; 8 -> 64 98
+// and 47, 17.7 and 16.2 (16 -> 64: 100 and 75, but 17.7 and 22.4).
+bool dx_by_pairs(const BwdArgs& b) {
+    return b.C_in <= (b.dt == HC_BF16 ? 32 : 8);
+}
+
 template <typename T>
-hc_status launch_act(const BwdArgs& b, const PrepArgs& prep, bool wide, T* dz, float* bpart,
-                     unsigned* status, cudaStream_t s) {
-    const dim3 grid((unsigned)(prep.act_blocks + prep.unit_blocks + prep.hist_blocks));
+hc_status launch_act(const BwdArgs& b, const PrepArgs& prep, bool wide, T* dz, int pitch,
+                     float* bpart, unsigned* status, cudaStream_t s) {
+    const dim3 grid((unsigned)(prep.act_blocks + prep.unit_blocks + prep.hist_blocks + prep.w_blocks));
     return launch_pdl(wide ? act_bwd_vec_kernel<T> : act_bwd_kernel<T>, grid, dim3(256), 0, s,
                       "act_bwd_kernel", (const T*)b.y, (const T*)b.dy, b.count,
-                      (long long)b.capacity, b.C_out, b.act, dz, bpart, prep, status);
+                      (long long)b.capacity, b.C_out, b.act, dz, pitch, bpart, prep, status);
 }
 
 }  // namespace
@@ -1876,9 +1944,15 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
     const int c_tiles = (b.C_in + BC - 1) / BC, o_tiles = (b.C_out + kTile - 1) / kTile;
     int G = (w_tc ? 1 : 2) * ctx->num_sms / (c_tiles * o_tiles);
     if (G < 1) G = 1;
-    // tap GEMM: P's rows padded to whole 16-byte chunks
+    // dgrad: P's rows padded to whole 16-byte chunks, and dz's and W's where
+    // the product needs it (bf16 off the tensor cores' alignment ran on CUDA cores
+    // otherwise: 64 -> 42, 41.9k rows, dx 130 us against 61)
     const int Cp = (b.C_in + vec - 1) / vec * vec;
-    const bool p_tc = bf && b.C_out % 8 == 0 && (uintptr_t)b.W % 16 == 0;
+    const bool pairs = b.dx && dx_by_pairs(b);
+    const bool by_taps = b.dx && !pairs;
+    const bool pad = by_taps && bf && (b.C_out % 8 != 0 || (uintptr_t)b.W % 16 != 0);
+    const int Cz = pairs || pad ? (b.C_out + vec - 1) / vec * vec : b.C_out;  // columns of dz
+    const size_t w_elems = pairs ? (size_t)b.L * Cp * Cz : pad ? (size_t)b.L * b.C_in * Cz : 0;
 
     const int slot_blocks = 2 * ctx->num_sms;
 
@@ -1889,17 +1963,18 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         if (wanted) total += (bytes + 255) / 256 * 256;
         return at;
     };
-    const size_t dz_at = take(true, (size_t)b.capacity * b.C_out * eb);
+    const size_t dz_at = take(true, (size_t)b.capacity * Cz * eb);
     const size_t bp_at = take(true, sizeof(float) * (size_t)act_blocks * b.C_out);
     const size_t part_at = take(b.dW, sizeof(float) * (size_t)c_tiles * o_tiles * (G + b.L) * BC * kTile);
     const size_t unit_at = take(b.dW, sizeof(int32_t) * (size_t)b.L * kUnits);
     const size_t ul_at = take(b.dW, sizeof(int2) * (size_t)capL);
     const size_t pos_at = take(b.dW, sizeof(int32_t) * (size_t)(b.L + 2));
     const size_t p_at = take(b.dx, (size_t)capL * Cp * eb);
-    const size_t ln_at = take(b.dx, sizeof(int32_t) * (size_t)capL);
-    const size_t le_at = take(b.dx, sizeof(int32_t) * (size_t)capL);
-    const size_t hist_at = take(b.dx, sizeof(int32_t) * (size_t)slot_blocks * b.L);
-    const size_t off_at = take(b.dx, sizeof(int32_t) * (size_t)(b.L + 1));
+    const size_t w_at = take(w_elems > 0, w_elems * eb);
+    const size_t ln_at = take(by_taps, sizeof(int32_t) * (size_t)capL);
+    const size_t le_at = take(by_taps, sizeof(int32_t) * (size_t)capL);
+    const size_t hist_at = take(by_taps, sizeof(int32_t) * (size_t)slot_blocks * b.L);
+    const size_t off_at = take(by_taps, sizeof(int32_t) * (size_t)(b.L + 1));
     uint8_t* ws = (uint8_t*)stream_workspace(s, total);
     if (!ws) return HC_ERR_CUDA;
     void* dz = ws + dz_at;
@@ -1908,7 +1983,7 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
     PrepArgs prep{};
     prep.act_blocks = (int)act_blocks;
     prep.unit_blocks = b.dW ? (b.L * kUnits + 7) / 8 : 0;
-    prep.hist_blocks = b.dx ? slot_blocks : 0;
+    prep.hist_blocks = by_taps ? slot_blocks : 0;
     prep.rb = b.rulebook;
     prep.L = b.L;
     prep.x_rows = b.x_rows;
@@ -1918,9 +1993,15 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
     prep.row_ptr = b.row_ptr;
     prep.taps = b.taps;
     prep.hist = (int32_t*)(ws + hist_at);
-    hc_status st = bf ? launch_act<__nv_bfloat16>(b, prep, act_wide, (__nv_bfloat16*)dz, bpart,
+    prep.w_blocks = pairs ? ((b.L * Cp + 31) / 32) * ((Cz + 31) / 32) : (int)((w_elems + 1023) / 1024);
+    prep.W = b.W;
+    prep.w_out = ws + w_at;
+    prep.C_in = b.C_in;
+    prep.Cp = pairs ? Cp : 0;
+    prep.Cz = Cz;
+    hc_status st = bf ? launch_act<__nv_bfloat16>(b, prep, act_wide, (__nv_bfloat16*)dz, Cz, bpart,
                                                   ctx->status, s)
-                      : launch_act<float>(b, prep, act_wide, (float*)dz, bpart, ctx->status, s);
+                      : launch_act<float>(b, prep, act_wide, (float*)dz, Cz, bpart, ctx->status, s);
     if (st != HC_OK) return st;
 
     if (b.dW) {
@@ -1932,6 +2013,7 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         w.L = b.L;
         w.C_in = b.C_in;
         w.C_out = b.C_out;
+        w.z_pitch = Cz;
         w.c_tiles = c_tiles;
         w.o_tiles = o_tiles;
         w.G = G;
@@ -1950,7 +2032,7 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         if (st != HC_OK) return st;
     }
     SlotArgs sl{};
-    if (b.dx) {
+    if (by_taps) {
         sl.row_ptr = b.row_ptr;
         sl.taps = b.taps;
         sl.x_rows = b.x_rows;
@@ -1988,41 +2070,55 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         if (st != HC_OK) return st;
     }
 
-    if (b.dx) {
+    if (!b.dx) return st;
+    void* const P = ws + p_at;
+    if (pairs) {
+        ConvArgs c{};  // P [rows][L * Cp] = dz W^T
+        c.x = dz;
+        c.count = b.count;
+        c.W = prep.w_out;
+        c.y = P;
+        c.capacity = c.x_rows = b.capacity;
+        c.B = 1;
+        c.V = b.capacity;
+        c.L = 1;
+        c.C_in = c.K = Cz;
+        c.C_out = b.L * Cp;
+        c.mode = kLinear;
+        c.act = HC_ACT_NONE;
+        st = dispatch_conv(ctx, c, b.dt, s);  // Cz whole chunks: needs no workspace
+    } else {
         TapGemmArgs g{};
         g.dz = dz;
-        g.W = b.W;
+        g.W = pad ? prep.w_out : b.W;
         g.slot_off = sl.slot_off;
         g.list_n = sl.list_n;
         g.list_e = sl.list_e;
-        g.P = ws + p_at;
+        g.P = P;
         g.L = b.L;
         g.C_in = b.C_in;
-        g.C_out = b.C_out;
+        g.C_out = Cz;
         g.Cp = Cp;
         g.status = ctx->status;
-        if (p_tc) {
+        if (bf) {
             g.c_tiles = (b.C_in + (b.C_in <= 64 ? 63 : 127)) / (b.C_in <= 64 ? 64 : 128);
             st = b.C_in <= 64 ? launch_tap_gemm_tc<64>(ctx, g, s) : launch_tap_gemm_tc<128>(ctx, g, s);
         } else {
             g.c_tiles = (b.C_in + kTgBN - 1) / kTgBN;
-            st = launch_pdl(bf ? tap_gemm_simt_kernel<__nv_bfloat16> : tap_gemm_simt_kernel<float>,
-                            dim3((unsigned)(2 * ctx->num_sms)), dim3(256), 0, s,
-                            "tap_gemm_simt_kernel", g);
+            st = launch_pdl(tap_gemm_simt_kernel, dim3((unsigned)(2 * ctx->num_sms)), dim3(256),
+                            0, s, "tap_gemm_simt_kernel", g);
         }
-        if (st != HC_OK) return st;
-        const int vec_ok = b.C_in % vec == 0 && (uintptr_t)b.dx % 16 == 0;
-        const long long blocks = ((long long)b.x_rows + kSegRows - 1) / kSegRows;
-        if (bf)
-            st = launch_pdl(seg_sum_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(256), 0, s,
-                            "seg_sum_kernel", (const __nv_bfloat16*)g.P, b.row_ptr, b.x_rows,
-                            b.C_in, Cp, capL, (__nv_bfloat16*)b.dx, vec_ok, ctx->status);
-        else
-            st = launch_pdl(seg_sum_kernel<float>, dim3((unsigned)blocks), dim3(256), 0, s,
-                            "seg_sum_kernel", (const float*)g.P, b.row_ptr, b.x_rows, b.C_in, Cp,
-                            capL, (float*)b.dx, vec_ok, ctx->status);
     }
-    return st;
+    if (st != HC_OK) return st;
+    const int vec_ok = b.C_in % vec == 0 && (uintptr_t)b.dx % 16 == 0;
+    const dim3 blocks((unsigned)(((long long)b.x_rows + kSegRows - 1) / kSegRows));
+    if (bf)
+        return launch_pdl(pairs ? seg_sum_kernel<__nv_bfloat16, true> : seg_sum_kernel<__nv_bfloat16, false>,
+                          blocks, dim3(256), 0, s, "seg_sum_kernel", (const __nv_bfloat16*)P, b.row_ptr,
+                          b.taps, b.x_rows, b.C_in, Cp, capL, (__nv_bfloat16*)b.dx, vec_ok, ctx->status);
+    return launch_pdl(pairs ? seg_sum_kernel<float, true> : seg_sum_kernel<float, false>, blocks, dim3(256),
+                      0, s, "seg_sum_kernel", (const float*)P, b.row_ptr, b.taps, b.x_rows, b.C_in, Cp,
+                      capL, (float*)b.dx, vec_ok, ctx->status);
 }
 
 }  // namespace hc
