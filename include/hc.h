@@ -352,7 +352,11 @@ hc_status hc_conv_rulebook_transpose(const int32_t* rulebook, const int32_t* cou
  * bf16: dW on tensor cores (tcgen05, fp32 accumulation); dz and the
  * per-tap products dz W^T are rounded to bf16 once before the input-gradient
  * sums. fp32: CUDA cores throughout. Every sum runs in a fixed order
- * (deterministic). Uses the library's per-stream workspace.
+ * (deterministic). Uses the library's per-stream workspace: a copy of dy in
+ * dt; for dx the per-tap products, capacity * L rows of C_in channels in dt
+ * (rounded up to 16 bytes), and 8 bytes per rulebook entry; for dW partial
+ * sums (about 64 KB per SM and per slot) and, without dx, 8 bytes per rulebook
+ * entry.
  */
 hc_status hc_sparse_conv_rulebook_bwd(const void* x, hc_dtype dt, int x_rows,
                                       const int32_t* rulebook, const int32_t* count, int capacity,

@@ -1967,9 +1967,10 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
     const size_t bp_at = take(true, sizeof(float) * (size_t)act_blocks * b.C_out);
     const size_t part_at = take(b.dW, sizeof(float) * (size_t)c_tiles * o_tiles * (G + b.L) * BC * kTile);
     const size_t unit_at = take(b.dW, sizeof(int32_t) * (size_t)b.L * kUnits);
-    const size_t ul_at = take(b.dW, sizeof(int2) * (size_t)capL);
     const size_t pos_at = take(b.dW, sizeof(int32_t) * (size_t)(b.L + 2));
     const size_t p_at = take(b.dx, (size_t)capL * Cp * eb);
+    // wgrad is done with its lists before P (at least 16 bytes an entry) is written
+    const size_t ul_at = b.dx ? p_at : take(b.dW, sizeof(int2) * (size_t)capL);
     const size_t w_at = take(w_elems > 0, w_elems * eb);
     const size_t ln_at = take(by_taps, sizeof(int32_t) * (size_t)capL);
     const size_t le_at = take(by_taps, sizeof(int32_t) * (size_t)capL);
