@@ -1003,15 +1003,21 @@ __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs
 // same runs; a block reads kSimtBatch taps of the lists at a time and
 // multiplies them kSimtBK at a time, the next rows in registers
 // while the current ones are multiplied. 64 channels of x by 128 of dz per
-// block, 4 x 8 per thread: 12 shared-memory words for 32 multiply-adds.
+// block, 4 x 8 per thread: 12 shared-memory words for 32 multiply-adds. With
+// up to 16 channels of x (BC 16) a quarter of the threads covers them, and the
+// four quarters take every fourth tap and add up at the end (with 64 the
+// padding was multiplied: 41.9k rows, every tap present, fp32 3 -> 64 160 us
+// and 80 us, 137 on tiles over all pairs; 12% of them 21 and 16 us, 45).
 constexpr int kSimtBK = 16;
 constexpr int kSimtBatch = 256;  // the block's threads: one entry each
-constexpr int kSimtBC = 64;
 
-template <typename T>
+template <typename T, int BC>
 __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
-    __shared__ float Xs[2][kSimtBK][kSimtBC];
-    __shared__ float Zs[2][kSimtBK][kTile];
+    constexpr int kParts = 64 / BC;                 // groups of threads, each with its taps
+    constexpr int kXper = kSimtBK * BC / 256;       // x values a thread loads
+    static_assert(BC == 64 || BC == 16, "4 x 8 outputs a thread");
+    __shared__ __align__(16) float Xs[2][kSimtBK][BC];
+    __shared__ __align__(16) float Zs[2][kSimtBK][kTile];
     __shared__ int s_j[kSimtBatch], s_n[kSimtBatch], red[8];
     extern __shared__ int s_pre[];  // [L * kUnits + 1]
     pdl_wait();
@@ -1032,9 +1038,10 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
                                  : ((T_ + a.G - 1) / a.G + kBK - 1) / kBK * kBK;
     }
     const long long urows = unit_rows(rows);
-    const int tx = t & 15, ty = t >> 4;  // outputs: c = ty * 4 .., o = tx * 4 .. and 64 + tx * 4 ..
-    // loads: x channel t % 64 of taps t / 64 + 4 i; dz channel t % 128 of taps t / 128 + 2 i
-    const int c = ct * kSimtBC + (t & 63), o = ot * kTile + (t & 127);
+    // outputs: c = ty * 4 .., o = tx * 4 .. and 64 + tx * 4 .., of taps part, + kParts, ..
+    const int tx = t & 15, ty = (t >> 4) % (BC / 4), part = (t >> 4) / (BC / 4);
+    // loads: x channel t % BC of taps t / BC + (256 / BC) i; dz channel t % 128 of taps t / 128 + 2 i
+    const int c = ct * BC + (t & (BC - 1)), o = ot * kTile + (t & 127);
     const bool c_ok = c < a.C_in, o_ok = o < a.C_out;
     int l = 0;
     for (long long pos = run.p0; pos < run.p1;) {
@@ -1053,11 +1060,11 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
                 s_n[t] = e.y - 1;
             }
             __syncthreads();
-            float xv[4], zv[8];
+            float xv[kXper], zv[8];
             auto fetch = [&](int k0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k = k0 + (t >> 6) + 4 * i;
+                for (int i = 0; i < kXper; ++i) {
+                    const int k = k0 + t / BC + (256 / BC) * i;
                     const int j = k < want ? s_j[k] : -1;
                     xv[i] = j >= 0 && c_ok ? to_f(x[(long long)j * a.C_in + c]) : 0.f;
                 }
@@ -1072,13 +1079,15 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
             int buf = 0;
             for (int k0 = 0; k0 < want; k0 += kSimtBK, buf ^= 1) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) Xs[buf][(t >> 6) + 4 * i][t & 63] = xv[i];
+                for (int i = 0; i < kXper; ++i)
+                    Xs[buf][t / BC + (256 / BC) * i][t & (BC - 1)] = xv[i];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) Zs[buf][(t >> 7) + 2 * i][t & 127] = zv[i];
                 __syncthreads();
                 if (k0 + kSimtBK < want) fetch(k0 + kSimtBK);
 #pragma unroll
-                for (int k = 0; k < kSimtBK; ++k) {
+                for (int kk = 0; kk < kSimtBK / kParts; ++kk) {
+                    const int k = kk * kParts + part;
                     const float4 xa = *reinterpret_cast<const float4*>(&Xs[buf][k][ty * 4]);
                     const float4 za = *reinterpret_cast<const float4*>(&Zs[buf][k][tx * 4]);
                     const float4 zb = *reinterpret_cast<const float4*>(&Zs[buf][k][64 + tx * 4]);
@@ -1092,13 +1101,36 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
             }
             __syncthreads();  // the list and the buffers are free
         }
-        float* dst = a.part + ((long long)blockIdx.y * (a.G + a.L) + g + l) * (kSimtBC * kTile);
+        if (kParts > 1) {  // the parts' sums onto the first's, in order
+            float* const sum = &Zs[0][0][0];  // [BC][kTile]
+            static_assert(kParts == 1 || BC * kTile <= 2 * kSimtBK * kTile, "a tile fits");
+            for (int p = 1; p < kParts; ++p) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float* d = dst + (ty * 4 + i) * kTile + tx * 4;
-            *reinterpret_cast<float4*>(d) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            *reinterpret_cast<float4*>(d + 64) =
-                make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int jj = 0; jj < 8; ++jj) {
+                        float& e = sum[(ty * 4 + i) * kTile + (jj / 4) * 64 + tx * 4 + jj % 4];
+                        if (part == p) e = acc[i][jj];
+                    }
+                __syncthreads();
+                if (part == 0)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int jj = 0; jj < 8; ++jj)
+                            acc[i][jj] += sum[(ty * 4 + i) * kTile + (jj / 4) * 64 + tx * 4 + jj % 4];
+                __syncthreads();
+            }
+        }
+        if (part == 0) {
+            float* dst = a.part + ((long long)blockIdx.y * (a.G + a.L) + g + l) * (BC * kTile);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float* d = dst + (ty * 4 + i) * kTile + tx * 4;
+                *reinterpret_cast<float4*>(d) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+                *reinterpret_cast<float4*>(d + 64) =
+                    make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+            }
         }
         pos = end;
     }
@@ -1940,7 +1972,7 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
     // wgrad: tensor cores for bf16 rows of whole 16-byte chunks; one CTA per
     // SM over all tiles (two on CUDA cores)
     const bool w_tc = bf && b.C_in % 8 == 0 && b.C_out % 8 == 0 && (uintptr_t)b.x % 16 == 0;
-    const int BC = w_tc && b.C_in > 64 ? 128 : 64;
+    const int BC = w_tc ? (b.C_in > 64 ? 128 : 64) : (b.C_in > 16 ? 64 : 16);
     const int c_tiles = (b.C_in + BC - 1) / BC, o_tiles = (b.C_out + kTile - 1) / kTile;
     int G = (w_tc ? 1 : 2) * ctx->num_sms / (c_tiles * o_tiles);
     if (G < 1) G = 1;
@@ -2028,8 +2060,10 @@ hc_status launch_conv_bwd(const DeviceCtx* ctx, const BwdArgs& b, cudaStream_t s
         if (w_tc)
             st = BC == 64 ? launch_wgrad_tc<64>(ctx, w, s) : launch_wgrad_tc<128>(ctx, w, s);
         else
-            st = launch_pdl(bf ? wgrad_simt_kernel<__nv_bfloat16> : wgrad_simt_kernel<float>, grid,
-                            dim3(256), pre, s, "wgrad_simt_kernel", w);
+            st = launch_pdl(bf ? (BC == 16 ? wgrad_simt_kernel<__nv_bfloat16, 16>
+                                           : wgrad_simt_kernel<__nv_bfloat16, 64>)
+                               : (BC == 16 ? wgrad_simt_kernel<float, 16> : wgrad_simt_kernel<float, 64>),
+                            grid, dim3(256), pre, s, "wgrad_simt_kernel", w);
         if (st != HC_OK) return st;
     }
     SlotArgs sl{};

@@ -1,6 +1,7 @@
 """The input gradient's two products (over the present taps, and with few input
-channels over all pairs) at the channel counts where they change and where rows
-of dz, W and P are padded, alone and with the other gradients, against the CPU
+channels over all pairs) and the weight gradient's two tiles on CUDA cores (16
+and 64 input channels) at the channel counts where they change and where rows of
+dz, W and P are padded, alone and with the other gradients, against the CPU
 oracle; a key outside the mapping is reported by both. Cases, tolerances: those
 of tests/test_gpu_bwd.py."""
 import pytest
@@ -18,7 +19,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,C_in,C_out", [
     ("bf16", 1, 64), ("bf16", 7, 42), ("bf16", 32, 10), ("bf16", 32, 64), ("bf16", 33, 42),
     ("bf16", 64, 1), ("bf16", 40, 66), ("bf16", 130, 42), ("f32", 1, 6), ("f32", 5, 64),
-    ("f32", 8, 20), ("f32", 9, 20), ("f32", 16, 3)])
+    ("f32", 8, 20), ("f32", 9, 20), ("f32", 16, 3), ("f32", 3, 130), ("bf16", 15, 70),
+    ("f32", 17, 130)])
 @pytest.mark.parametrize("layout", [oracle.LAYOUT_DENSE, oracle.LAYOUT_COMPACT])
 def test_bwd_channels(dtype, C_in, C_out, layout):
     c = _case(C_in * 100 + C_out, 3, 260, 7, C_in, C_out, dtype, layout, oracle.ACT_ELU)

@@ -104,3 +104,18 @@ def test_input_gradient_of_few_or_odd_channels():
                                 (torch.float32, 3, 64, 0.5)):
         t, base = dx_us(ci, co, dtype), dx_us(64, 64, dtype)
         assert t < most * base, (dtype, ci, co, t, base)
+
+
+def test_weight_gradient_of_few_channels():
+    """3 of 64 input channels in fp32 are not as much work as 64 (0.99 of their time
+    with one tile width)."""
+    L, n = 9, 41920
+    rb, c = neighbours(L, n), count(n)
+
+    def dW_us(ci):
+        x, y, dy = (torch.randn(s, device="cuda") for s in ((n, ci), (n, 64), (n, 64)))
+        dW = torch.empty((L * ci, 64), device="cuda")
+        return us(lambda: hc.hc_sparse_conv_rulebook_bwd(x, rb, c, dW, y, dy, hc.HC_ACT_ELU, None,
+                                                         None, None, dW, None))
+    few, many = dW_us(3), dW_us(64)
+    assert few < 0.75 * many, (few, many)
