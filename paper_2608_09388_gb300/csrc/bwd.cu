@@ -811,10 +811,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs
     const int ct = (int)blockIdx.y % a.c_tiles, ot = (int)blockIdx.y / a.c_tiles;
     const Run run(s_pre, a.L, a.G, g);
     if (g == 0 && blockIdx.y == 0 && (int)threadIdx.x <= a.L + 1) {
-        const int T = s_pre[a.L * kUnits];
+        const long long T = s_pre[a.L * kUnits];
         a.slot_pos[threadIdx.x] = (int)threadIdx.x <= a.L
                                       ? s_pre[threadIdx.x * kUnits]
-                                      : ((T + a.G - 1) / a.G + kBK - 1) / kBK * kBK;
+                                      : (int)(((T + a.G - 1) / a.G + kBK - 1) / kBK * kBK);
     }
 
     if (warp < kProducerWarps) {
@@ -1033,9 +1033,9 @@ __global__ void __launch_bounds__(256, 2) wgrad_simt_kernel(const WgradArgs a) {
     const Run run(s_pre, a.L, a.G, g);
     const int t = threadIdx.x;
     if (g == 0 && blockIdx.y == 0 && t <= a.L + 1) {
-        const int T_ = s_pre[a.L * kUnits];
+        const long long T_ = s_pre[a.L * kUnits];
         a.slot_pos[t] = t <= a.L ? s_pre[t * kUnits]
-                                 : ((T_ + a.G - 1) / a.G + kBK - 1) / kBK * kBK;
+                                 : (int)(((T_ + a.G - 1) / a.G + kBK - 1) / kBK * kBK);
     }
     const long long urows = unit_rows(rows);
     // outputs: c = ty * 4 .., o = tx * 4 .. and 64 + tx * 4 .., of taps part, + kParts, ..
@@ -1325,7 +1325,7 @@ __device__ __forceinline__ void slot_tiles(const int32_t* slot_off, int L, int* 
     const int lane = threadIdx.x & 31;
     const int off = lane < L ? __ldg(slot_off + lane) : 0;
     const int nxt = lane < L ? __ldg(slot_off + lane + 1) : 0;
-    const int tiles = (nxt - off + BM - 1) / BM;
+    const int tiles = (int)(((long long)nxt - off + BM - 1) / BM);
     int x = tiles;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1474,8 +1474,8 @@ __global__ void __launch_bounds__(kTapThreads, 1)
                 const int end = s_off[l + 1];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const int e = first + (t >> 3) + 16 * i;
-                    n[i] = e < end ? __ldg(a.list_n + e) : -1;
+                    const int r = (t >> 3) + 16 * i;
+                    n[i] = r < end - first ? __ldg(a.list_n + first + r) : -1;
                 }
             }
         };
@@ -1600,8 +1600,8 @@ __global__ void __launch_bounds__(kTapThreads, 1)
             if (w >= items) return;
             int first;
             locate(w, l, first, c0_next);
-            const int i = first + ew * 32 + lane;
-            e_next = i < s_off[l + 1] ? __ldg(a.list_e + i) : -1;
+            const int r = ew * 32 + lane;
+            e_next = r < s_off[l + 1] - first ? __ldg(a.list_e + first + r) : -1;
         };
         entry(blockIdx.x);
         for (long long w = blockIdx.x; w < items; w += gridDim.x, ++lt) {
@@ -1687,12 +1687,12 @@ __global__ void __launch_bounds__(256, 2) tap_gemm_simt_kernel(const TapGemmArgs
         const int c0 = (int)(w - (long long)tile * a.c_tiles) * kTgBN;
         while (s_tile[l + 1] <= tile) ++l;
         const int first = s_off[l] + (tile - s_tile[l]) * kTgBM, end = s_off[l + 1];
-        if (t < kTgBM) s_e[t] = first + t < end ? __ldg(a.list_e + first + t) : -1;
+        if (t < kTgBM) s_e[t] = t < end - first ? __ldg(a.list_e + first + t) : -1;
         long long za[4], wb[2];  // first element of this thread's rows, -1: none
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int e = first + ra + 4 * i;
-            const int n = e < end ? __ldg(a.list_n + e) : -1;
+            const int r = ra + 4 * i;
+            const int n = r < end - first ? __ldg(a.list_n + first + r) : -1;
             za[i] = n >= 0 ? (long long)n * a.C_out : -1;
         }
 #pragma unroll
@@ -1833,12 +1833,12 @@ __global__ void __launch_bounds__(256, 6)
         float acc[VEC];
 #pragma unroll
         for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
-        for (int e = s_ptr[i]; e < e1; e += 4) {
+        for (int e = s_ptr[i]; e < e1; e = e1 - e > 4 ? e + 4 : e1) {
             uint4 v[4];
             bool use[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                use[q] = e + q < e1;
+                use[q] = q < e1 - e;
                 if (!kKeys) {
                     if (use[q]) v[q] = ld_hint(P + (long long)(e + q) * Cp + col, let_go);
                 } else if (use[q]) {
@@ -1850,7 +1850,7 @@ __global__ void __launch_bounds__(256, 6)
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (kKeys ? use[q] : e + q < e1) {
+                if (kKeys ? use[q] : q < e1 - e) {
                     const T* p = reinterpret_cast<const T*>(&v[q]);
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) acc[k] += to_f(p[k]);
