@@ -746,11 +746,6 @@ struct WgradCfg {
     static size_t smem_bytes(int L) { return 1024 + kPre + sizeof(int) * ((size_t)L * kUnits + 1); }
 };
 
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 template <int BC>
 __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs a) {
     using C = WgradCfg<BC>;
@@ -947,8 +942,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) wgrad_tc_kernel(const WgradArgs
                     const uint32_t z_st = base + st * C::kStageBytes, x_st = z_st + 2 * kAtomBytes;
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
-                        const uint64_t zd = desc_sw128(z_st + k * 16 * 128, kAtomBytes, 1024);
-                        const uint64_t xd = desc_sw128(x_st + k * 16 * 128, kAtomBytes, 1024);
+                        const uint64_t zd = smem_desc_sw128(z_st + k * 16 * 128, kAtomBytes, 1024);
+                        const uint64_t xd = smem_desc_sw128(x_st + k * 16 * 128, kAtomBytes, 1024);
                         tc_mma_bf16(tmem_base + (uint32_t)(acc * BC), zd, xd, C::kIdesc,
                                     first ? 0u : 1u);
                         first = false;
@@ -1375,29 +1370,6 @@ struct TapCfg {
 // possible (evict last) and let go with their read (evict first), and dx, which
 // nothing here reads again, streams past it (training step at 64 x 10475, 25%
 // density, 128 MB of P: 268.8 -> 264 us).
-__device__ __forceinline__ uint64_t l2_keep() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ uint64_t l2_let_go() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void st_hint(void* p, uint4 v, uint64_t pol) {
-    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(v.x),
-                 "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
-                 : "memory");
-}
-__device__ __forceinline__ uint4 ld_hint(const void* p, uint64_t pol) {
-    uint4 v;
-    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p), "l"(pol));
-    return v;
-}
-
 constexpr int kTapEpilogueWarps = 8;  // 4-7 and 10-13: half of the columns each
 constexpr int kTapThreads = (kIndexWarp + 1 + 4) * 32;
 
@@ -1570,8 +1542,8 @@ __global__ void __launch_bounds__(kTapThreads, 1)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         tc_mma_bf16(tmem_base + (uint32_t)(acc * BN),
-                                    desc_sw128(a_st + k * 32, 16, 1024),
-                                    desc_sw128(b_st + k * 32, 16, 1024), C::kIdesc,
+                                    smem_desc_sw128(a_st + k * 32, 16, 1024),
+                                    smem_desc_sw128(b_st + k * 32, 16, 1024), C::kIdesc,
                                     (kb | k) != 0 ? 1u : 0u);
                     tc_commit(empty_bar(st));
                     if (++st == kStages) {
@@ -1593,7 +1565,7 @@ __global__ void __launch_bounds__(kTapThreads, 1)
         const int half = warp < kMmaWarp ? 0 : 1;      // columns half * BN / 2 ..
         const uint32_t stage = base + C::kEpi + (half * 4 + (warp < kMmaWarp ? ew : warp - 10)) * 2048;
         __nv_bfloat16* P = static_cast<__nv_bfloat16*>(a.P);
-        const uint64_t keep = l2_keep();
+        const uint64_t keep = l2_evict_last_policy();
         int lt = 0, l = 0, c0 = 0, c0_next = 0;
         long long e_next = -1;  // the next item's, read one item ahead
         auto entry = [&](long long w) {
@@ -1817,7 +1789,7 @@ __global__ void __launch_bounds__(256, 6)
                 if (col + k < C_in) dst[k] = from_f<T>(v[k]);
         }
     };
-    const uint64_t let_go = l2_let_go();
+    const uint64_t let_go = l2_evict_first_policy();
     const int nb = s_nb;
     if (nb < n) {
         const float zero[VEC] = {};

@@ -137,14 +137,6 @@ struct Cfg {
     }
 };
 
-// Shared-memory matrix descriptor: start address, leading and stride byte
-// offsets (>> 4), fixed version bits 46-48 = 0b001, 128-byte swizzle (2 at
-// bits 61-63), base offset 0 (stage buffers are 1024-byte aligned).
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 // Epilogue of one 32-column chunk of a warp's 32 output rows: activation,
 // bf16 rounding (RNE), then the stores. Lane i holds row i's 32 fp32 sums
 // (bias included) in r. The rows go through a 2 KB shared buffer (16-byte

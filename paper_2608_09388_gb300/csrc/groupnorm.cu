@@ -112,24 +112,6 @@ struct Chunk<__nv_bfloat16, 8> {
     }
 };
 
-// 16-byte accesses with an L2 evict-first policy (last use of a line).
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ uint4 ld_ef(const void* p, uint64_t pol) {
-    uint4 v;
-    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ void st_ef(void* p, uint4 v, uint64_t pol) {
-    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(v.x),
-                 "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
-                 : "memory");
-}
 template <typename Raw>
 __device__ __forceinline__ Raw as_raw(uint4 v) {
     return *reinterpret_cast<const Raw*>(&v);
@@ -462,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
         for (int i = 0; i < kBatch; ++i)
             if (top - (long long)i * l.rpp >= 0)
-                cur[i] = as_raw<Raw>(ld_ef(x + row_at(top - (long long)i * l.rpp), pol));
+                cur[i] = as_raw<Raw>(ld_hint(x + row_at(top - (long long)i * l.rpp), pol));
         __syncthreads();  // s_mu / s_inv of the previous segment have been read
         if (part_rows > 0) {
             // whole blocks [w0, w1) of the frame's rows [p0, p1], and its
@@ -539,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) {
                 const long long r = r0 - step - (long long)i * l.rpp;
-                if (r >= 0) nxt[i] = as_raw<Raw>(ld_ef(x + row_at(r), pol));
+                if (r >= 0) nxt[i] = as_raw<Raw>(ld_hint(x + row_at(r), pol));
             }
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) {
@@ -556,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                     T* dst = y + row_at(r);
                     Raw packed;
                     CK::store(reinterpret_cast<T*>(&packed), v);
-                    st_ef(dst, as_u4(packed), pol);
+                    st_hint(dst, as_u4(packed), pol);
                 }
             }
 #pragma unroll

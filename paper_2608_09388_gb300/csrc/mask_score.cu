@@ -83,13 +83,6 @@ __device__ __forceinline__ int tile_index(int tm, int tn, int nt) {
     return tm * nt - tm * (tm - 1) / 2 + (tn - tm);
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle, version bits 46-48 =
-// 0b001 (the stage buffers are 1024-byte aligned).
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 // ---------------------------------------------------------------- bf16: tcgen05
 // Warps 0-3 load both operand tiles of a stage: thread t owns 16-byte chunk
 // column t % (TILE/8) of the TILE feature columns (atom cc / 8, chunk cc % 8
@@ -224,10 +217,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1) gram_tc_kernel(const GramArgs a
                 const uint32_t b_st = diag ? a_st : sB + s * kOpBytes;
 #pragma unroll
                 for (int k = 0; k < kBK / 16; ++k) {
-                    const uint64_t bd = desc_sw128(b_st + k * 16 * 128, kAtom, 1024);
+                    const uint64_t bd = smem_desc_sw128(b_st + k * 16 * 128, kAtom, 1024);
 #pragma unroll
                     for (int h = 0; h < Cf::kHalves; ++h) {
-                        const uint64_t ad = desc_sw128(a_st + h * 2 * kAtom + k * 16 * 128, kAtom, 1024);
+                        const uint64_t ad = smem_desc_sw128(a_st + h * 2 * kAtom + k * 16 * 128, kAtom, 1024);
                         tc_mma_bf16(tmem_base + h * TILE, ad, bd, kIdesc, (kb | k) != 0 ? 1u : 0u);
                     }
                 }
