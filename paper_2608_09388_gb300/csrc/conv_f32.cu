@@ -340,7 +340,10 @@ hc_status launch_cfg(const DeviceCtx* ctx, const ConvArgs& a, cudaStream_t s) {
 // several slots a step (41.9k rows, 9 slots, 3 -> 64: 44 us here, 22 there at
 // every tap present, 12.4 and 10.3 at 15%; 32 slots 129 and 30 us): below 16
 // channels, or 8 with the 128-output tiles (8 -> 128: 23 us here, 27 there at
-// half of the taps present).
+// half of the taps present). A sparse layer above that is taken whatever
+// its mask, which only the device knows: with every tap present the tiles would
+// be ahead up to 48 channels (16 -> 64: 49 us here, 44 there; 45 -> 64: 112 and
+// 88), at half of the taps (21 and 26; 43 and 66) and below it is not close.
 // The dense layer has no absent tap to skip besides, so it is not taken where
 // channels come element by element (45 -> 42 over 42k rows: 90 us there, 123
 // here), where an odd number of 64-wide tiles above one splits the outputs
